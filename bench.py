@@ -51,7 +51,8 @@ sys.path.insert(0, ROOT)
 
 N_DEFAULT = 8192
 METRIC = "TFLOP/s & % of tensor peak, matmul/conv2d, BF16/FP8 vs FP32 at stated error"
-GEMM_SOURCES = ("paper_2307_16080_gb300/csrc/k_tc_gemm.cu", "paper_2307_16080_gb300/csrc/tc_ptx.cuh")
+GEMM_SOURCES = ("paper_2307_16080_gb300/csrc/tc_gemm.cuh", "paper_2307_16080_gb300/csrc/k_tc_gemm.cu",
+                "paper_2307_16080_gb300/csrc/tc_ptx.cuh")
 FLUSH_BYTES = 256 << 20
 
 

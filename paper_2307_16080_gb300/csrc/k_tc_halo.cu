@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
             const int ncol = p.F - col0 < 32 ? p.F - col0 : 32;
             if (p.ew.n) {
               // the program runs out of line on a local buffer (see below)
-              float buf[32];
+              __align__(16) float buf[32];
 #pragma unroll
               for (int j = 0; j < 32; ++j) {
                 float xv = v[j];
@@ -453,7 +453,9 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
                 buf[j] = xv;
               }
               ew_apply(p.ew, buf, ncol, orow_off + col0);
-              for (int j = 0; j < ncol; ++j) dh[j] = __float2bfloat16_rn(buf[j]);
+              if (p.c_vec32 && ncol == 32) store32_bf16_v8(dh, buf);
+              else
+                for (int j = 0; j < ncol; ++j) dh[j] = __float2bfloat16_rn(buf[j]);
             } else {
 #pragma unroll
               for (int j = 0; j < 32; ++j) {
@@ -483,7 +485,7 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
             // buffer so the program reads its operands (which may alias O)
             // before the store and v[] is not live across the call.
             const int ncol = p.F - col0 < 32 ? p.F - col0 : 32;
-            float buf[32];
+            __align__(16) float buf[32];
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
               float xv = v[j];
@@ -495,7 +497,9 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
               buf[j] = xv;
             }
             ew_apply(p.ew, buf, ncol, orow_off + col0);
-            for (int j = 0; j < ncol; ++j) dst[j] = buf[j];
+            if (p.c_vec32 && ncol == 32) store32_f32_v8(dst, buf);
+            else
+              for (int j = 0; j < ncol; ++j) dst[j] = buf[j];
           } else if (p.c_vec32 && p.beta == 0.f && col0 + 32 <= p.F) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
