@@ -4,15 +4,21 @@
 // "linalg-matmul") and, through an implicit im2col A-operand, the NHWC/HWCF
 // convolution of Sec. 4.1 Listing "2dnchwconv".  The loop nest is tiled the
 // way Sec. 4.3 tunes it -- output tiles per CTA, a reduction depth per step --
-// but written for sm_103: 256 threads per CTA, BMxBN tiles of 64 or 128,
-// BK = 16, a double-buffered shared-memory ring fed by 128-bit loads,
-// register blocking of (BM/16)x(BN/16) outputs per thread, and FFMA in FP32.
+// but written for sm_103: tiles of 128 x 128, 128 x 64 or 64 x 64, BK = 16, a
+// four-stage shared-memory ring fed by asynchronous copies, register blocking
+// of 8 x 8 (8 x 4) outputs per thread, and FP32 FMAs.
 //
-// Split-K: the reduction range is cut into `splits` slices (grid z); each
-// slice writes its partial tile to the workspace and a second kernel sums the
-// slices in a fixed order with a warp-shuffle tree, then applies the epilogue.
+// Split-K, two ways.  On request (schedule split_k): the reduction range is
+// cut into `splits` slices (grid z); each slice writes its partial tile to the
+// workspace and a second kernel sums the slices in a fixed order with a
+// warp-shuffle tree, then applies the epilogue.  By the built-in rule, for
+// outputs with too few tiles: the CTAs of a cluster each take a slice of K and
+// add their tiles through distributed shared memory, in a fixed order, with
+// no workspace and no second kernel.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "nk_internal.cuh"
@@ -23,14 +29,19 @@ namespace {
 constexpr int BK = 16;
 constexpr int THREADS = 256;
 
-// Operand loading modes.
-enum AMode { A_SCALAR = 0, A_KVEC = 1, A_MVEC = 2, A_CONV_VEC = 3, A_CONV_SCALAR = 4 };
-enum BMode { B_SCALAR = 0, B_NVEC = 1, B_KVEC = 2 };
+// How an operand tile reaches shared memory: along k (k contiguous in memory),
+// along the tile's other dimension, or (conv) by the im2col gather along k; in
+// 4-byte copies, or in 16-byte ones where the operand's alignment allows them.
+// 16-byte copies along k store a tile of A as [m][k]; the others store [k][m]
+// and [k][n], 4-byte copies along k scattering a row of k.
+enum LoadMode { L_K = 0, L_MN = 1, L_MN16 = 2, L_CONV = 3, L_K16 = 4, L_CONV16 = 5 };
 
 struct KArgs {
   SimtGemm p;
   int k_chunk;      // reduction length handled by one grid-z slice
   float* partial;   // [splits][M][N] or null
+  int csplit;       // CTAs of a cluster that share one tile's reduction (1: none)
+  int tiles_n;
 };
 
 // Implicit im2col element A[m,k] of the convolution (0 outside the input);
@@ -55,46 +66,325 @@ __device__ __forceinline__ float conv_a(const SimtGemm& p, int m, int k, int64_t
   return p.A[*off];
 }
 
-// Four consecutive k (same tap, since C % 4 == 0) of conv row m; *off as
-// for conv_a, for the first of the four.
-__device__ __forceinline__ float4 conv_a4(const SimtGemm& p, int m, int k, int64_t* off) {
-  const ConvGeom& g = p.conv;
-  int ow = m % g.ow;
-  int t = m / g.ow;
-  int oh = t % g.oh;
-  int n = t / g.oh;
-  int c = k % g.c;
-  int tap = k / g.c;
-  int kw = tap % g.kw;
-  int kh = tap / g.kw;
-  int ih = oh * g.sh + kh * g.dh - g.pt;
-  int iw = ow * g.sw + kw * g.dw - g.pl;
-  if (ih < 0 || ih >= g.h || iw < 0 || iw >= g.w) {
-    *off = -1;
-    return make_float4(0.f, 0.f, 0.f, 0.f);
+__device__ __forceinline__ void cp4(uint32_t dst, const float* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp16(uint32_t dst, const float* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Epilogue of four consecutive outputs (m, nb..nb+3).
+__device__ __forceinline__ void finish4(const SimtGemm& p, int m, int nb, const float (&acc)[4]) {
+  float v[4];
+  float* crow = p.C + (int64_t)m * p.scm;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int n = nb + j;
+    float o = p.alpha * acc[j];
+    if (n < p.N) {
+      if (p.beta != 0.f) o = fmaf(p.beta, crow[(int64_t)n * p.scn], o);
+      if (p.bias) o += __ldg(p.bias + (p.bias_on_m ? m : n));
+      if (p.relu) o = (o > 0.f || o != o) ? o : 0.f;
+    }
+    v[j] = o;
   }
-  *off = n * g.sin_n + ih * g.sin_h + iw * g.sin_w + c;
-  return __ldg(reinterpret_cast<const float4*>(p.A + *off));
+  if (p.scn == 1 && nb + 3 < p.N && ((reinterpret_cast<uintptr_t>(crow + nb) & 15) == 0)) {
+    *reinterpret_cast<float4*>(crow + nb) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (nb + j < p.N) crow[(int64_t)(nb + j) * p.scn] = v[j];
+  }
 }
 
-// Prologue on four loaded values whose offsets are off, off+d, off+2d, off+3d.
-__device__ __forceinline__ void pro4(const EwProg& e, float4& v, int64_t off, int64_t d) {
-  v.x = ew_run(e, v.x, off);
-  v.y = ew_run(e, v.y, off + d);
-  v.z = ew_run(e, v.z, off + 2 * d);
-  v.w = ew_run(e, v.w, off + 3 * d);
+// What bounds it: the FMA pipes (128 lanes a cycle and SM), so everything else
+// has to fit in the issue slots beside them.  FMAs are issued two to an
+// instruction on pairs of columns (fma.rn.f32x2, each half rounded as fmaf:
+// the sums are bitwise those of a scalar loop); operands come through a ring
+// of asynchronous copies, which need no registers, no second pass to store
+// and no alignment -- a row of odd length loads as fast as an aligned one;
+// rows past M (columns past N) read a clamped row whose results are dropped,
+// so only the end of K is predicated.  A loop of these FMAs over resident tiles
+// reaches 66 TFLOP/s (scalar FMAs 60); the kernel 56 at 4096^3 (54 before).
+// Odd row lengths, which took scalar loads: 1531 x 2047 x 1021 230 -> 150 us.
+template <int BM, int BN, int T, int AM, int BMD>
+__global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __grid_constant__ KArgs args) {
+  constexpr int S = 4;                  // stages
+  constexpr int TY = BM / 8, TX = T / TY, TN = BN / TX;
+  constexpr bool CONV = AM == L_CONV || AM == L_CONV16;
+  constexpr bool AMK = AM == L_CONV16 || AM == L_K16;   // A is stored [m][k]
+  constexpr int A_LD = AMK ? BK + 4 : BM + 4, B_LD = BN + 4;
+  constexpr int A_FL = AMK ? BM * A_LD : BK * A_LD;
+  constexpr int STAGE = A_FL + BK * B_LD;
+  constexpr int KV = T == 256 ? 2 : 4;   // k values of A in registers at a time (256 threads: 128 registers each)
+  static_assert(TN == 8 || TN == 4, "8 x 8 or 8 x 4 outputs per thread");
+  static_assert(S * STAGE >= BM * BN, "a cluster's partial tiles reuse the ring");
+  extern __shared__ __align__(16) float smem[];
+  __shared__ int row_off[BM], row_hw[BM];   // conv: offset of a row's first tap, and its (ih, iw)
+  nk::pdl_wait();      // earlier kernels on the stream have finished
+  nk::pdl_trigger();
+  const SimtGemm& p = args.p;
+  const int tid = threadIdx.x;
+  const int tx = tid % TX, ty = tid / TX;
+  const int cs = args.csplit;
+  const int crank = cs > 1 ? (int)(blockIdx.x % cs) : 0;
+  const int m0 = blockIdx.y * BM;
+  const int n0 = (cs > 1 ? (int)(blockIdx.x / cs) : (int)blockIdx.x) * BN;
+  const int kbeg = (cs > 1 ? crank : (int)blockIdx.z) * args.k_chunk;
+  const int kend = min(p.K, kbeg + args.k_chunk);
+  const int ntiles = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
+
+  if constexpr (CONV) {
+    const ConvGeom& g = p.conv;
+    for (int r = tid; r < BM; r += T) {
+      const int m = min(m0 + r, p.M - 1);
+      const int ow = m % g.ow, q = m / g.ow, oh = q % g.oh, n = q / g.oh;
+      const int ih = oh * g.sh - g.pt, iw = ow * g.sw - g.pl;
+      row_off[r] = (int)(n * g.sin_n + ih * g.sin_h + iw * g.sin_w);
+      row_hw[r] = (ih << 16) | (iw & 0xffff);
+    }
+    __syncthreads();
+  }
+  // per-thread load positions, fixed for the whole loop
+  const int lk = tid % BK, lr = tid / BK;          // along k: this thread's k and first row
+  constexpr int LR = T / BK;
+  constexpr int KC = (AM == L_K16 || AM == L_CONV16) ? 4 : 1;   // k values a copy of A brings
+  const int ak = tid % (BK / KC) * KC, ar = tid / (BK / KC);
+  constexpr int AR = T * KC / BK;
+  auto load_tile = [&](int t) {
+    const int k0 = kbeg + t * BK;
+    const uint32_t sa = sbase + (uint32_t)((t % S) * STAGE * 4);
+    const uint32_t sb = sa + (uint32_t)(A_FL * 4);
+    auto cpa = [](uint32_t dst, const float* src, bool ok) {
+      if constexpr (KC == 4) cp16(dst, src, ok);
+      else cp4(dst, src, ok);
+    };
+    if constexpr (CONV) {
+      const ConvGeom& g = p.conv;
+      const int k = k0 + ak;
+      const bool ok = k < kend;
+      const int kc = ok ? k : 0;
+      const int tap = kc / g.c, c = kc - tap * g.c;
+      const int kh = tap / g.kw, kw = tap - kh * g.kw;
+      const int dh = kh * g.dh, dw = kw * g.dw;
+      const int d = (int)(dh * g.sin_h + dw * g.sin_w) + c;
+#pragma unroll
+      for (int i = 0; i < BM / AR; ++i) {
+        const int r = ar + i * AR;
+        const int hw = row_hw[r];
+        const int ih = (hw >> 16) + dh, iw = (int)(short)(hw & 0xffff) + dw;
+        const bool in = ok && (unsigned)ih < (unsigned)g.h && (unsigned)iw < (unsigned)g.w;
+        cpa(sa + (uint32_t)((AMK ? r * A_LD + ak : ak * A_LD + r) * 4), p.A + (in ? row_off[r] + d : 0), in);
+      }
+    } else if constexpr (AM == L_K || AM == L_K16) {
+      const int k = k0 + ak;
+      const bool ok = k < kend;
+      const float* src = p.A + (int64_t)(ok ? k : 0) * p.sak;
+#pragma unroll
+      for (int i = 0; i < BM / AR; ++i) {
+        const int r = ar + i * AR;
+        cpa(sa + (uint32_t)((AMK ? r * A_LD + ak : ak * A_LD + r) * 4), src + (int64_t)min(m0 + r, p.M - 1) * p.sam, ok);
+      }
+    } else if constexpr (AM == L_MN) {
+      const int r = tid % BM;
+#pragma unroll
+      for (int i = 0; i < BK * BM / T; ++i) {
+        const int kk = tid / BM + i * (T / BM);
+        const bool ok = k0 + kk < kend;
+        cp4(sa + (uint32_t)((kk * A_LD + r) * 4),
+            p.A + (int64_t)(ok ? k0 + kk : 0) * p.sak + (int64_t)min(m0 + r, p.M - 1) * p.sam, ok);
+      }
+    } else {
+      const int r = tid % (BM / 4) * 4;
+#pragma unroll
+      for (int i = 0; i < BK * BM / 4 / T; ++i) {
+        const int kk = tid / (BM / 4) + i * (T / (BM / 4));
+        const bool ok = k0 + kk < kend;
+        cp16(sa + (uint32_t)((kk * A_LD + r) * 4), p.A + (int64_t)(ok ? k0 + kk : 0) * p.sak + min(m0 + r, p.M - 4), ok);
+      }
+    }
+    if constexpr (BMD == L_K) {
+      const int k = k0 + lk;
+      const bool ok = k < kend;
+      const float* src = p.B + (int64_t)(ok ? k : 0) * p.sbk;
+#pragma unroll
+      for (int i = 0; i < BN / LR; ++i) {
+        const int c = lr + i * LR;
+        cp4(sb + (uint32_t)((lk * B_LD + c) * 4), src + (int64_t)min(n0 + c, p.N - 1) * p.sbn, ok);
+      }
+    } else if constexpr (BMD == L_MN) {
+      const int c = tid % BN;
+#pragma unroll
+      for (int i = 0; i < BK * BN / T; ++i) {
+        const int kk = tid / BN + i * (T / BN);
+        const bool ok = k0 + kk < kend;
+        cp4(sb + (uint32_t)((kk * B_LD + c) * 4),
+            p.B + (int64_t)(ok ? k0 + kk : 0) * p.sbk + (int64_t)min(n0 + c, p.N - 1) * p.sbn, ok);
+      }
+    } else {
+      const int c = tid % (BN / 4) * 4;
+#pragma unroll
+      for (int i = 0; i < BK * BN / 4 / T; ++i) {
+        const int kk = tid / (BN / 4) + i * (T / (BN / 4));
+        const bool ok = k0 + kk < kend;
+        cp16(sb + (uint32_t)((kk * B_LD + c) * 4), p.B + (int64_t)(ok ? k0 + kk : 0) * p.sbk + min(n0 + c, p.N - 4), ok);
+      }
+    }
+  };
+
+  f2 acc[8][TN / 2];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < TN / 2; ++j) acc[i][j] = f2_set(0.f);
+
+#pragma unroll
+  for (int t = 0; t < S - 1; ++t) {
+    if (t < ntiles) load_tile(t);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  for (int t = 0; t < ntiles; ++t) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+    __syncthreads();   // tile t has landed for every thread, and tile t - 1 is read: its slot is free
+    if (t + S - 1 < ntiles) load_tile(t + S - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* As = smem + (t % S) * STAGE;
+    const float* Bs = As + A_FL;
+    auto step = [&](int kk, const float (&a)[8]) {
+      f2 b[TN / 2];
+#pragma unroll
+      for (int h = 0; h < TN / 4; ++h) {
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(Bs + kk * B_LD + h * (BN / 2) + tx * 4);
+        b[2 * h].v = q.x;
+        b[2 * h + 1].v = q.y;
+      }
+      f2 aa[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) aa[i] = f2_set(a[i]);
+#pragma unroll
+      for (int j = 0; j < TN / 2; ++j)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[i][j] = f2_fma(aa[i], b[j], acc[i][j]);
+    };
+    if constexpr (AMK) {
+#pragma unroll
+      for (int kq = 0; kq < BK; kq += KV) {
+        float av[8][KV];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float* src = As + (ty + TY * i) * A_LD + kq;
+          if constexpr (KV == 4) {
+            const float4 q = *reinterpret_cast<const float4*>(src);
+            av[i][0] = q.x; av[i][1] = q.y; av[i][2] = q.z; av[i][3] = q.w;
+          } else {
+            const float2 q = *reinterpret_cast<const float2*>(src);
+            av[i][0] = q.x; av[i][1] = q.y;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < KV; ++e) {
+          float a[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) a[i] = av[i][e];
+          step(kq + e, a);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int kk = 0; kk < BK; ++kk) {
+        const float4 a0 = *reinterpret_cast<const float4*>(As + kk * A_LD + ty * 4);
+        const float4 a1 = *reinterpret_cast<const float4*>(As + kk * A_LD + BM / 2 + ty * 4);
+        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        step(kk, a);
+      }
+    }
+  }
+  // the tile row of this thread's output i
+  auto row_of = [&](int i) { return AMK ? ty + TY * i : (i / 4) * (BM / 2) + ty * 4 + (i % 4); };
+
+  if (cs > 1) {
+    // Every CTA of the cluster leaves its partial tile in its ring (whose last
+    // copies have landed and been read); then each finishes a share of the
+    // tile's rows, adding the slices in rank order.
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int h = 0; h < TN / 4; ++h) {
+        const int r = row_of(i), c = h * (BN / 2) + tx * 4;
+        ulonglong2 q;
+        q.x = acc[i][2 * h].v;
+        q.y = acc[i][2 * h + 1].v;
+        *reinterpret_cast<ulonglong2*>(smem + r * BN + c) = q;
+      }
+    cluster_barrier();
+    const int share = BM / cs;
+    for (int e = tid; e < share * (BN / 4); e += T) {
+      const int r = crank * share + e / (BN / 4), c = (e % (BN / 4)) * 4;
+      float4 sum = ld_cluster4(cluster_map(sbase + (uint32_t)((r * BN + c) * 4), 0));
+      for (int q = 1; q < cs; ++q) {
+        const float4 v = ld_cluster4(cluster_map(sbase + (uint32_t)((r * BN + c) * 4), (uint32_t)q));
+        sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+      }
+      if (m0 + r < p.M && n0 + c < p.N) {
+        const float v[4] = {sum.x, sum.y, sum.z, sum.w};
+        finish4(p, m0 + r, n0 + c, v);
+      }
+    }
+    cluster_barrier();   // no CTA leaves while another may still read its tile
+    return;
+  }
+  // Epilogue: partial tile to the workspace, or the fused epilogue to C.
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int m = m0 + row_of(i);
+    if (m >= p.M) continue;
+#pragma unroll
+    for (int h = 0; h < TN / 4; ++h) {
+      const int nb = n0 + h * (BN / 2) + tx * 4;
+      float v[4];
+      f2_get(acc[i][2 * h], v[0], v[1]);
+      f2_get(acc[i][2 * h + 1], v[2], v[3]);
+      if (args.partial) {
+        float* dst = args.partial + ((int64_t)blockIdx.z * p.M + m) * p.N;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (nb + j < p.N) dst[nb + j] = v[j];
+      } else if (nb < p.N) {
+        finish4(p, m, nb, v);
+      }
+    }
+  }
 }
 
-// FUSED: the variant that runs prologue / epilogue programs (instantiated
-// with the scalar load modes only); the plain variants carry no call.
-template <int RM, int RN, int AM, int BMD, bool FUSED>
-__global__ void __launch_bounds__(THREADS, 2) simt_gemm_kernel(const __grid_constant__ KArgs args) {
+// The kernel that runs prologue / epilogue programs: scalar loads of any
+// layout into registers, where a prologue can change them (256 threads, 64 or
+// 128 square tiles, a double-buffered tile).
+template <int RM, int RN, bool CONV>
+__global__ void __launch_bounds__(THREADS, 2) simt_fused_kernel(const __grid_constant__ KArgs args) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
   constexpr int BM = 64 * RM;
   constexpr int BN = 64 * RN;
-  constexpr int APAD = 4;
-  constexpr int A_LD = BM + APAD;
+  constexpr int A_LD = BM + 4;
   constexpr int NA = BM * BK / THREADS;   // scalars of A each thread loads per tile
   constexpr int NB = BN * BK / THREADS;
   __shared__ __align__(16) float As[2][BK][A_LD];
@@ -113,144 +403,48 @@ __global__ void __launch_bounds__(THREADS, 2) simt_gemm_kernel(const __grid_cons
   float rb[NB];
 
   auto load_a = [&](int k0) {
-    if constexpr (AM == A_KVEC || AM == A_CONV_VEC) {
 #pragma unroll
-      for (int j = 0; j < NA / 4; ++j) {
-        int L = tid + j * THREADS;
-        int row = L / 4, kq = (L % 4) * 4;
-        int m = m0 + row, k = k0 + kq;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (m < p.M && k < kend) {
-          int64_t off = (int64_t)m * p.sam + k;
-          if constexpr (AM == A_KVEC)
-            v = __ldg(reinterpret_cast<const float4*>(p.A + off));
-          else
-            v = conv_a4(p, m, k, &off);
-          if (FUSED && p.pro_a.n && off >= 0) pro4(p.pro_a, v, off, 1);
-        }
-        ra[4 * j + 0] = v.x; ra[4 * j + 1] = v.y; ra[4 * j + 2] = v.z; ra[4 * j + 3] = v.w;
+    for (int j = 0; j < NA; ++j) {
+      int L = tid + j * THREADS;
+      int row = L % BM, kk = L / BM;
+      int m = m0 + row, k = k0 + kk;
+      float v = 0.f;
+      if (m < p.M && k < kend) {
+        int64_t off = (int64_t)m * p.sam + (int64_t)k * p.sak;
+        if constexpr (CONV) v = conv_a(p, m, k, &off);
+        else v = p.A[off];
+        if (p.pro_a.n && off >= 0) v = ew_run(p.pro_a, v, off);
       }
-    } else if constexpr (AM == A_MVEC) {
-#pragma unroll
-      for (int j = 0; j < NA / 4; ++j) {
-        int L = tid + j * THREADS;
-        int kk = L / (BM / 4), mq = (L % (BM / 4)) * 4;
-        int m = m0 + mq, k = k0 + kk;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (m < p.M && k < kend) {
-          v = __ldg(reinterpret_cast<const float4*>(p.A + (int64_t)k * p.sak + m));
-          if (FUSED && p.pro_a.n) pro4(p.pro_a, v, (int64_t)k * p.sak + m, 1);
-        }
-        ra[4 * j + 0] = v.x; ra[4 * j + 1] = v.y; ra[4 * j + 2] = v.z; ra[4 * j + 3] = v.w;
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < NA; ++j) {
-        int L = tid + j * THREADS;
-        int row = L % BM, kk = L / BM;
-        int m = m0 + row, k = k0 + kk;
-        float v = 0.f;
-        if (m < p.M && k < kend) {
-          int64_t off = (int64_t)m * p.sam + (int64_t)k * p.sak;
-          if constexpr (AM == A_CONV_SCALAR) v = conv_a(p, m, k, &off);
-          else v = p.A[off];
-          if (FUSED && p.pro_a.n && off >= 0) v = ew_run(p.pro_a, v, off);
-        }
-        ra[j] = v;
-      }
+      ra[j] = v;
     }
   };
   auto store_a = [&](int buf) {
-    if constexpr (AM == A_KVEC || AM == A_CONV_VEC) {
 #pragma unroll
-      for (int j = 0; j < NA / 4; ++j) {
-        int L = tid + j * THREADS;
-        int row = L / 4, kq = (L % 4) * 4;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) As[buf][kq + i][row] = ra[4 * j + i];
-      }
-    } else if constexpr (AM == A_MVEC) {
-#pragma unroll
-      for (int j = 0; j < NA / 4; ++j) {
-        int L = tid + j * THREADS;
-        int kk = L / (BM / 4), mq = (L % (BM / 4)) * 4;
-        *reinterpret_cast<float4*>(&As[buf][kk][mq]) =
-            make_float4(ra[4 * j], ra[4 * j + 1], ra[4 * j + 2], ra[4 * j + 3]);
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < NA; ++j) {
-        int L = tid + j * THREADS;
-        As[buf][L / BM][L % BM] = ra[j];
-      }
+    for (int j = 0; j < NA; ++j) {
+      int L = tid + j * THREADS;
+      As[buf][L / BM][L % BM] = ra[j];
     }
   };
   auto load_b = [&](int k0) {
-    if constexpr (BMD == B_NVEC) {
 #pragma unroll
-      for (int j = 0; j < NB / 4; ++j) {
-        int L = tid + j * THREADS;
-        int kk = L / (BN / 4), nq = (L % (BN / 4)) * 4;
-        int n = n0 + nq, k = k0 + kk;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (n < p.N && k < kend) {
-          v = __ldg(reinterpret_cast<const float4*>(p.B + (int64_t)k * p.sbk + n));
-          if (FUSED && p.pro_b.n) pro4(p.pro_b, v, (int64_t)k * p.sbk + n, 1);
-        }
-        rb[4 * j + 0] = v.x; rb[4 * j + 1] = v.y; rb[4 * j + 2] = v.z; rb[4 * j + 3] = v.w;
+    for (int j = 0; j < NB; ++j) {
+      int L = tid + j * THREADS;
+      int col = L % BN, kk = L / BN;
+      int n = n0 + col, k = k0 + kk;
+      float v = 0.f;
+      if (n < p.N && k < kend) {
+        const int64_t off = (int64_t)k * p.sbk + (int64_t)n * p.sbn;
+        v = p.B[off];
+        if (p.pro_b.n) v = ew_run(p.pro_b, v, off);
       }
-    } else if constexpr (BMD == B_KVEC) {
-#pragma unroll
-      for (int j = 0; j < NB / 4; ++j) {
-        int L = tid + j * THREADS;
-        int col = L / 4, kq = (L % 4) * 4;
-        int n = n0 + col, k = k0 + kq;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (n < p.N && k < kend) {
-          v = __ldg(reinterpret_cast<const float4*>(p.B + (int64_t)n * p.sbn + k));
-          if (FUSED && p.pro_b.n) pro4(p.pro_b, v, (int64_t)n * p.sbn + k, 1);
-        }
-        rb[4 * j + 0] = v.x; rb[4 * j + 1] = v.y; rb[4 * j + 2] = v.z; rb[4 * j + 3] = v.w;
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < NB; ++j) {
-        int L = tid + j * THREADS;
-        int col = L % BN, kk = L / BN;
-        int n = n0 + col, k = k0 + kk;
-        float v = 0.f;
-        if (n < p.N && k < kend) {
-          const int64_t off = (int64_t)k * p.sbk + (int64_t)n * p.sbn;
-          v = p.B[off];
-          if (FUSED && p.pro_b.n) v = ew_run(p.pro_b, v, off);
-        }
-        rb[j] = v;
-      }
+      rb[j] = v;
     }
   };
   auto store_b = [&](int buf) {
-    if constexpr (BMD == B_NVEC) {
 #pragma unroll
-      for (int j = 0; j < NB / 4; ++j) {
-        int L = tid + j * THREADS;
-        int kk = L / (BN / 4), nq = (L % (BN / 4)) * 4;
-        *reinterpret_cast<float4*>(&Bs[buf][kk][nq]) =
-            make_float4(rb[4 * j], rb[4 * j + 1], rb[4 * j + 2], rb[4 * j + 3]);
-      }
-    } else if constexpr (BMD == B_KVEC) {
-#pragma unroll
-      for (int j = 0; j < NB / 4; ++j) {
-        int L = tid + j * THREADS;
-        int col = L / 4, kq = (L % 4) * 4;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) Bs[buf][kq + i][col] = rb[4 * j + i];
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < NB; ++j) {
-        int L = tid + j * THREADS;
-        Bs[buf][L / BN][L % BN] = rb[j];
-      }
+    for (int j = 0; j < NB; ++j) {
+      int L = tid + j * THREADS;
+      Bs[buf][L / BN][L % BN] = rb[j];
     }
   };
 
@@ -323,7 +517,7 @@ __global__ void __launch_bounds__(THREADS, 2) simt_gemm_kernel(const __grid_cons
           if (p.beta != 0.f) o = fmaf(p.beta, p.C[(int64_t)m * p.scm + (int64_t)n * p.scn], o);
           if (p.bias) o += p.bias[p.bias_on_m ? m : n];
           if (p.relu) o = (o > 0.f || o != o) ? o : 0.f;
-          if (FUSED && p.ew.n) o = ew_run(p.ew, o, (int64_t)m * p.scm + (int64_t)n * p.scn);
+          if (p.ew.n) o = ew_run(p.ew, o, (int64_t)m * p.scm + (int64_t)n * p.scn);
         }
         v[j] = o;
       }
@@ -376,38 +570,106 @@ __global__ void splitk_reduce_kernel(const __grid_constant__ SplitReduce r, int 
   }
 }
 
-template <int RM, int RN, int AM>
+template <int BM, int BN, int T, int AM, int BMD>
+nk_status launch_kernel(const KArgs& a, dim3 grid, cudaStream_t st) {
+  auto kern = simt_gemm_kernel<BM, BN, T, AM, BMD>;
+  constexpr bool amk = AM == L_K16 || AM == L_CONV16;
+  constexpr int smem = 4 * ((amk ? BM * (BK + 4) : BK * (BM + 4)) + BK * (BN + 4)) * (int)sizeof(float);
+  if constexpr (smem + 2 * BM * (int)sizeof(int) > 48 * 1024) {
+    static std::atomic<bool> set[64];   // per device; setting it twice is harmless
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !set[dev].load(std::memory_order_relaxed)) {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(simt_gemm_kernel)");
+      if (dev >= 0 && dev < 64) set[dev].store(true, std::memory_order_relaxed);
+    }
+  }
+  const cudaError_t e = nk::launch_k(kern, grid, dim3(T), smem, st, a.csplit, a);
+  if (e != cudaSuccess) return cuda_fail(e, "launch simt_gemm_kernel");
+  return check_launch("simt_gemm_kernel");
+}
+
+template <int BM, int BN, int T, int AM>
 nk_status launch_b(const KArgs& a, int bmode, dim3 grid, cudaStream_t st) {
   switch (bmode) {
-    case B_NVEC: (void)nk::launch_k(simt_gemm_kernel<RM, RN, AM, B_NVEC, false>, dim3(grid), dim3(THREADS), 0, st, 1, a); break;
-    case B_KVEC: (void)nk::launch_k(simt_gemm_kernel<RM, RN, AM, B_KVEC, false>, dim3(grid), dim3(THREADS), 0, st, 1, a); break;
-    default: (void)nk::launch_k(simt_gemm_kernel<RM, RN, AM, B_SCALAR, false>, dim3(grid), dim3(THREADS), 0, st, 1, a); break;
+    case L_K: return launch_kernel<BM, BN, T, AM, L_K>(a, grid, st);
+    case L_MN: return launch_kernel<BM, BN, T, AM, L_MN>(a, grid, st);
+    default: return launch_kernel<BM, BN, T, AM, L_MN16>(a, grid, st);
   }
-  return check_launch("simt_gemm_kernel");
 }
 
-// Programs present: scalar loads of any layout, FUSED kernel.
-template <int RM, int RN>
-nk_status launch_fused(const KArgs& a, dim3 grid, cudaStream_t st) {
-  if (a.p.is_conv)
-    (void)nk::launch_k(simt_gemm_kernel<RM, RN, A_CONV_SCALAR, B_SCALAR, true>, dim3(grid), dim3(THREADS), 0, st, 1, a);
-  else
-    (void)nk::launch_k(simt_gemm_kernel<RM, RN, A_SCALAR, B_SCALAR, true>, dim3(grid), dim3(THREADS), 0, st, 1, a);
-  return check_launch("simt_gemm_kernel");
-}
-
-template <int RM, int RN>
+template <int BM, int BN, int T>
 nk_status launch_a(const KArgs& a, int amode, int bmode, dim3 grid, cudaStream_t st) {
   switch (amode) {
-    case A_KVEC: return launch_b<RM, RN, A_KVEC>(a, bmode, grid, st);
-    case A_MVEC: return launch_b<RM, RN, A_MVEC>(a, bmode, grid, st);
-    case A_CONV_VEC: return launch_b<RM, RN, A_CONV_VEC>(a, bmode, grid, st);
-    case A_CONV_SCALAR: return launch_b<RM, RN, A_CONV_SCALAR>(a, bmode, grid, st);
-    default: return launch_b<RM, RN, A_SCALAR>(a, bmode, grid, st);
+    case L_K: return launch_b<BM, BN, T, L_K>(a, bmode, grid, st);
+    case L_K16:   // 256 threads have no registers for [m][k] (2629 us against 2460 at 4096^3)
+      if constexpr (T == 256) return launch_b<BM, BN, T, L_K>(a, bmode, grid, st);
+      else return launch_b<BM, BN, T, L_K16>(a, bmode, grid, st);
+    case L_MN: return launch_b<BM, BN, T, L_MN>(a, bmode, grid, st);
+    case L_MN16: return launch_b<BM, BN, T, L_MN16>(a, bmode, grid, st);
+    case L_CONV16:
+      return bmode == L_MN16 ? launch_kernel<BM, BN, T, L_CONV16, L_MN16>(a, grid, st)
+                             : launch_kernel<BM, BN, T, L_CONV16, L_MN>(a, grid, st);
+    default:   // a convolution's filters are row-major [K][F]
+      return bmode == L_MN16 ? launch_kernel<BM, BN, T, L_CONV, L_MN16>(a, grid, st)
+                             : launch_kernel<BM, BN, T, L_CONV, L_MN>(a, grid, st);
   }
+}
+
+// Programs present: the register-loading kernel.
+template <int RM, int RN>
+nk_status launch_fused(const KArgs& a, dim3 grid, cudaStream_t st) {
+  if (a.p.is_conv) (void)nk::launch_k(simt_fused_kernel<RM, RN, true>, grid, dim3(THREADS), 0, st, 1, a);
+  else (void)nk::launch_k(simt_fused_kernel<RM, RN, false>, grid, dim3(THREADS), 0, st, 1, a);
+  return check_launch("simt_fused_kernel");
 }
 
 inline bool al16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+// The built-in tile, and the CTAs that share a tile's reduction: the smallest
+// predicted time over the tiles and clusters of 1 to 8.  An SM works through
+// its units (tiles x slices) at the rate the tile's shape reaches, each unit
+// costs about a microsecond to fill and drain, and a cluster's exchange 1.6;
+// clusters of eight 128-row tiles pack badly.  The constants are fitted to
+// every combination timed on 23 shapes (products from 64^3 to 4096^3 and eight
+// convolutions), where the choice is 1.3 % off the best on average and 11 % at
+// worst.  Examples, us (tile / cluster): 256^3 64x64 / 1 12.3, / 8 5.3; 1024^3
+// 128x128 / 1 103, / 4 53; 1531 x 2047 x 1021 128x128 / 1 194, / 4 150;
+// 8x56x56x64 3x3 64x64 / 1 71, 128x64 / 2 52.
+struct Choice {
+  int bm, bn, csplit;
+};
+Choice choose(int M, int N, int K, int sms, bool may_split) {
+  struct Tile {
+    int bm, bn, resident;
+    double gflop_us;   // per SM
+  };
+  static const Tile kTiles[] = {{128, 128, 2, 0.366}, {128, 64, 3, 0.359}, {64, 64, 2, 0.355}};
+  Choice best{128, 128, 1};
+  double best_t = 1e30;
+  for (const Tile& t : kTiles) {
+    const int64_t tm = (M + t.bm - 1) / t.bm;
+    if (tm > 65535 && t.bm < 128) continue;   // grid.y
+    for (int cs = 1; cs <= (may_split ? 8 : 1) && (cs == 1 || cs * BK <= K); cs *= 2) {
+      const int64_t units = tm * ((N + t.bn - 1) / t.bn) * cs;
+      // units of the busiest SM: whole ones while all are resident at once,
+      // then the average and about half a set in the last wave
+      const double u = units <= (int64_t)sms * t.resident ? (double)((units + sms - 1) / sms)
+                                                          : (double)units / sms + 0.59 * t.resident;
+      const double warps = u * (t.bn == 128 ? 8 : 4);
+      const double fill = warps < 8 ? 0.575 : warps < 12 ? 0.864 : 1.0;   // too few to keep the FMA pipes busy
+      const double kc = ((K + cs - 1) / cs + BK - 1) / BK * BK;
+      const double pack = t.bm == 128 ? (cs == 8 ? 1.276 : cs == 4 ? 0.915 : 1.0) : 1.0;
+      const double us = u * (2e-6 * t.bm * t.bn * kc * pack / (t.gflop_us * fill) + 1.064) + (cs > 1 ? 1.642 : 0.0);
+      if (us < best_t) {
+        best_t = us;
+        best = {t.bm, t.bn, cs};
+      }
+    }
+  }
+  return best;
+}
 
 }  // namespace
 
@@ -418,7 +680,7 @@ size_t simt_gemm_ws(int M, int N, int splits) {
 nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws_bytes,
                     cudaStream_t st) {
   if (p.M <= 0 || p.N <= 0) return NK_OK;
-  if (tile != 64 && tile != 128) return fail(NK_ERR_INVALID_ARG, "SIMT tile must be 64 or 128");
+  if (tile != 0 && tile != 64 && tile != 128) return fail(NK_ERR_INVALID_ARG, "SIMT tile must be 64 or 128");
   if (splits < 1 || splits > 32) return fail(NK_ERR_INVALID_ARG, "split_k must be in [1, 32]");
   KArgs a;
   a.p = p;
@@ -428,37 +690,54 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
   splits = p.K > 0 ? (p.K + kc - 1) / kc : 1;
   a.k_chunk = kc;
   a.partial = nullptr;
+  a.csplit = 1;
+  a.tiles_n = 0;
   if (splits > 1) {
     if (!ws || ws_bytes < simt_gemm_ws(p.M, p.N, splits))
       return fail(NK_ERR_WORKSPACE, "split-K needs %zu bytes of workspace",
                   simt_gemm_ws(p.M, p.N, splits));
     a.partial = static_cast<float*>(ws);
   }
-  // Pick the load modes from the layout and alignment.
-  int amode, bmode;
-  if (p.is_conv) {
-    const ConvGeom& g = p.conv;
-    bool vec = (g.c % 4 == 0) && g.sin_n % 4 == 0 && g.sin_h % 4 == 0 && g.sin_w % 4 == 0 &&
-               al16(p.A);
-    amode = vec ? A_CONV_VEC : A_CONV_SCALAR;
-  } else if (p.sak == 1 && p.sam % 4 == 0 && p.K % 4 == 0 && al16(p.A)) {
-    amode = A_KVEC;
-  } else if (p.sam == 1 && p.sak % 4 == 0 && p.M % 4 == 0 && al16(p.A)) {
-    amode = A_MVEC;
+  // The gather keeps a pixel's offset in 32 bits and its position in 16.
+  const ConvGeom& cg = p.conv;
+  const bool far = p.is_conv && (cg.h + cg.pt + cg.kh * cg.dh > 32000 || cg.w + cg.pl + cg.kw * cg.dw > 32000 ||
+                                 cg.oh * (int64_t)cg.sh > 32000 || cg.ow * (int64_t)cg.sw > 32000 ||
+                                 cg.n * cg.sin_n + cg.h * cg.sin_h + cg.w * cg.sin_w >= INT32_MAX / 2);
+  if (p.pro_a.n || p.pro_b.n || p.ew.n || far) {
+    if (tile == 0) tile = (int64_t)((p.M + 127) / 128) * ((p.N + 127) / 128) < 152 ? 64 : 128;
+    const dim3 grid((p.N + tile - 1) / tile, (p.M + tile - 1) / tile, splits);
+    if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "M too large for the SIMT grid");
+    const nk_status s = tile == 128 ? launch_fused<2, 2>(a, grid, st) : launch_fused<1, 1>(a, grid, st);
+    if (s != NK_OK || splits == 1) return s;
   } else {
-    amode = A_SCALAR;
+    // Pick the load modes from the layout and alignment.
+    int amode, bmode;
+    if (p.is_conv)
+      amode = cg.c % 4 == 0 && cg.sin_n % 4 == 0 && cg.sin_h % 4 == 0 && cg.sin_w % 4 == 0 && al16(p.A) ? L_CONV16 : L_CONV;
+    else if (p.sak == 1 && p.sam % 4 == 0 && p.K % 4 == 0 && al16(p.A)) amode = L_K16;
+    else if (p.sam == 1 && p.sak != 1) amode = p.sak % 4 == 0 && p.M % 4 == 0 && al16(p.A) ? L_MN16 : L_MN;
+    else amode = L_K;
+    if (p.sbn == 1) bmode = p.sbk % 4 == 0 && p.N % 4 == 0 && al16(p.B) ? L_MN16 : L_MN;
+    else bmode = L_K;
+    int bm = tile, bn = tile;
+    if (tile == 0) {
+      int sms = 0;
+      const nk_status s = require_device(&sms);
+      if (s != NK_OK) return s;
+      const Choice c = choose(p.M, p.N, p.K, sms, splits == 1);
+      bm = c.bm;
+      bn = c.bn;
+      a.csplit = c.csplit;
+      if (a.csplit > 1) a.k_chunk = ((p.K + a.csplit - 1) / a.csplit + BK - 1) / BK * BK;
+    }
+    a.tiles_n = (p.N + bn - 1) / bn;
+    const dim3 grid(a.tiles_n * a.csplit, (p.M + bm - 1) / bm, splits);
+    if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "M too large for the SIMT grid");
+    const nk_status s = bn == 128   ? launch_a<128, 128, 256>(a, amode, bmode, grid, st)
+                        : bm == 128 ? launch_a<128, 64, 128>(a, amode, bmode, grid, st)
+                                    : launch_a<64, 64, 128>(a, amode, bmode, grid, st);
+    if (s != NK_OK || splits == 1) return s;
   }
-  if (p.sbn == 1 && p.sbk % 4 == 0 && p.N % 4 == 0 && al16(p.B)) bmode = B_NVEC;
-  else if (p.sbk == 1 && p.sbn % 4 == 0 && p.K % 4 == 0 && al16(p.B)) bmode = B_KVEC;
-  else bmode = B_SCALAR;
-  dim3 grid((p.N + tile - 1) / tile, (p.M + tile - 1) / tile, splits);
-  if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "M too large for the SIMT grid");
-  nk_status s;
-  if (p.pro_a.n || p.pro_b.n || p.ew.n)
-    s = tile == 128 ? launch_fused<2, 2>(a, grid, st) : launch_fused<1, 1>(a, grid, st);
-  else
-    s = tile == 128 ? launch_a<2, 2>(a, amode, bmode, grid, st) : launch_a<1, 1>(a, amode, bmode, grid, st);
-  if (s != NK_OK || splits == 1) return s;
   SplitReduce r{};
   r.partial = a.partial;
   r.splits = splits;

@@ -253,9 +253,7 @@ nk_status plan_matmul(const nk_tensor* A, const nk_tensor* B, const nk_tensor* C
   P.total = 0;
   if (prec == NK_PREC_F32) {
     int split = P.sched.split_k > 0 ? P.sched.split_k : 1;
-    int tile = P.sched.tile_m > 0 ? P.sched.tile_m : 128;
-    if (P.sched.tile_m == 0 && (int64_t)((P.M + 127) / 128) * ((P.N + 127) / 128) < 152) tile = 64;
-    P.sched.tile_m = P.sched.tile_n = tile;
+    P.sched.tile_n = P.sched.tile_m;   // 0: simt_gemm chooses
     P.sched.tile_k = 16;
     P.sched.cluster = 1;
     P.sched.stages = 2;
@@ -742,7 +740,7 @@ nk_status nk_conv2d_nhwc_hwcf(const nk_tensor* I, const nk_tensor* W, nk_tensor*
   p.alpha = 1.f; p.beta = E.accumulate ? 1.f : 0.f; p.relu = E.relu;
   p.is_conv = 1; p.conv = g;
   p.ew = ew; p.pro_a = pro_i; p.pro_b = pro_w;
-  int tile = sched && sched->tile_m > 0 ? sched->tile_m : 64;
+  int tile = sched && sched->tile_m > 0 ? sched->tile_m : 0;   // 0: simt_gemm chooses
   int split = sched && sched->split_k > 0 ? sched->split_k : 1;
   return simt_gemm(p, tile, split, ws, ws_bytes, static_cast<cudaStream_t>(stream));
 }

@@ -136,7 +136,7 @@ struct SimtGemm {
   EwProg pro_a, pro_b;   // prologues on the loaded A / B (offsets from A, B; conv: from I)
 };
 
-// tile: 128 or 64 (square CTA tile); splits >= 1.  When splits > 1 the
+// tile: 128 or 64 (square CTA tile), or 0 for the built-in choice; splits >= 1.  When splits > 1 the
 // partial sums go to `ws` ([splits][M][N] FP32) and a reduce pass applies
 // the epilogue.
 nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws_bytes,
