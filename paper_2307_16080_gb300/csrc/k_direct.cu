@@ -158,8 +158,16 @@ __device__ __forceinline__ void load_segment(const float* src, int64_t sIh, int 
     if (SEG >= 4 && (reinterpret_cast<uintptr_t>(q) & 15) == 0) {
       const float4 a = __ldg(reinterpret_cast<const float4*>(q));
       x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+      if constexpr (SEG == 6) {
+        const float2 b = __ldg(reinterpret_cast<const float2*>(q + 4));
+        x[4] = b.x; x[5] = b.y;
+      } else if constexpr (SEG == 8) {
+        const float4 b = __ldg(reinterpret_cast<const float4*>(q + 4));
+        x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+      } else {
 #pragma unroll
-      for (int j = 4; j < SEG; ++j) x[j] = __ldg(q + j);
+        for (int j = 4; j < SEG; ++j) x[j] = __ldg(q + j);
+      }
     } else {
 #pragma unroll
       for (int j = 0; j < SEG; ++j) x[j] = __ldg(q + j);
@@ -251,96 +259,167 @@ __global__ void __launch_bounds__(128) direct_rows_kernel(const __grid_constant_
   }
 }
 
-// Epilogue and store of 4 consecutive outputs of one row and channel.
-__device__ __forceinline__ void store4(const Direct& p, float* dst, int wo, float b, const float (&a)[4]) {
-  float v[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    float o = a[j];
-    if (p.beta != 0.f && wo + j < p.OW) o = fmaf(p.beta, dst[j], o);
-    o += b;
-    if (p.relu) o = (o > 0.f || o != o) ? o : 0.f;
-    v[j] = o;
-  }
-  const uintptr_t ad = reinterpret_cast<uintptr_t>(dst);
-  if (wo + 3 < p.OW && (ad & 15) == 0) {
-    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-  } else if (wo + 3 < p.OW && (ad & 7) == 0) {
-    *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
-    *reinterpret_cast<float2*>(dst + 2) = make_float2(v[2], v[3]);
+// Stores a warp's 128 consecutive outputs of one row and channel, four a lane,
+// to a row that starts s floats before a 16-byte boundary (the same s for the
+// whole warp) or ends inside the warp.  A lane stores its last 4 - s values
+// and its neighbour's first s as one aligned 16-byte word, so the warp writes
+// whole sectors; the ends of the row, and lane 0's first s values, go out one
+// by one.  Out of line: the unrolled loop keeps the two common cases.
+__device__ __noinline__ void store_shifted(float* dst, int s, int wo, int OW, float v0, float v1, float v2, float v3) {
+  const int lane = threadIdx.x & 31;
+  const float n0 = __shfl_down_sync(0xffffffffu, v0, 1);
+  const float n1 = __shfl_down_sync(0xffffffffu, v1, 1);
+  const float n2 = __shfl_down_sync(0xffffffffu, v2, 1);
+  if ((s == 0 || lane < 31) && wo + s + 3 < OW) {
+    *reinterpret_cast<float4*>(dst + s) =
+        make_float4(s == 0 ? v0 : s == 1 ? v1 : s == 2 ? v2 : v3, s == 0 ? v1 : s == 1 ? v2 : s == 2 ? v3 : n0,
+                    s == 0 ? v2 : s == 1 ? v3 : s == 2 ? n0 : n1, s == 0 ? v3 : s == 1 ? n0 : s == 2 ? n1 : n2);
   } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (wo + j < p.OW) dst[j] = v[j];
+    if (s <= 0 && wo < OW) dst[0] = v0;
+    if (s <= 1 && wo + 1 < OW) dst[1] = v1;
+    if (s <= 2 && wo + 2 < OW) dst[2] = v2;
+    if (wo + 3 < OW) dst[3] = v3;
+  }
+  if (s && (lane == 0 || wo + s - 1 >= OW)) {   // no lane before this one stored these
+    if (wo < OW) dst[0] = v0;
+    if (s > 1 && wo + 1 < OW) dst[1] = v1;
+    if (s > 2 && wo + 2 < OW) dst[2] = v2;
   }
 }
 
 // One input channel: output row o lives in accumulator slot o % KH while
-// input rows o .. o+KH-1 arrive; it is stored after the last of them.
-template <int KH, int KW, int CO_G>
+// input rows o .. o+KH-1 arrive; it is stored after the last of them.  The
+// next input row's loads are in flight while a row is used.
+//
+// What bounds it is issue slots, not HBM (an input row feeds KH x KW x CO FMAs
+// per output column, beside the loads' and stores' bookkeeping), so CO is the
+// exact number of output channels of the thread, PLAIN leaves accumulate and
+// ReLU out, and range and alignment are settled once per thread where they can
+// be.  16 x 1280 x 1280, 3 x 3, 1 -> 3 channels (418 MB): 330 instructions per
+// warp and row, four channels computed for three and 8-byte stores on every
+// other row took 123 us; now 84 us.
+template <int KH, int KW, int CO, bool PLAIN>
 __global__ void __launch_bounds__(128) direct_stream_kernel(const __grid_constant__ Direct p, int rpt) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
   constexpr int SEG = 4 + KW - 1;
   constexpr int TAPS = KH * KW;
+  const int lane = threadIdx.x & 31;
   const int wo = blockIdx.x * 512 + threadIdx.x * 4;
   const int ho0 = blockIdx.y * rpt;
-  const int groups = (p.CO + CO_G - 1) / CO_G;
+  const int groups = (p.CO + CO - 1) / CO;
   const int n = blockIdx.z / groups;
-  const int co0 = (blockIdx.z % groups) * CO_G;
-  const int ncog = min(CO_G, p.CO - co0);
-  if (wo >= p.OW || ho0 >= p.OH) return;
+  const int co0 = (blockIdx.z % groups) * CO;
+  const int ncog = min(CO, p.CO - co0);
+  if (wo - lane * 4 >= p.OW || ho0 >= p.OH) return;   // whole warps: the stores shuffle
   const int rows = min(rpt, p.OH - ho0);
-  float w[CO_G][TAPS];
+  float w[CO][TAPS];
 #pragma unroll
-  for (int c = 0; c < CO_G; ++c)
+  for (int c = 0; c < CO; ++c)
 #pragma unroll
     for (int t = 0; t < TAPS; ++t) w[c][t] = c < ncog ? __ldg(p.Kr + (int64_t)(co0 + c) * TAPS + t) : 0.f;
-  float bias[CO_G];
+  float bias[CO];
 #pragma unroll
-  for (int c = 0; c < CO_G; ++c) bias[c] = (p.bias && c < ncog) ? __ldg(p.bias + co0 + c) : 0.f;
-  float acc[KH][CO_G][4];
+  for (int c = 0; c < CO; ++c) bias[c] = (p.bias && c < ncog) ? __ldg(p.bias + co0 + c) : 0.f;
+  // Accumulators of the KH output rows under way.  A row's first tap row
+  // overwrites its slot, so the rows above the first output row (o < 0) leave
+  // nothing behind, and those past the last are never stored.
+  float acc[KH][CO][4];
 #pragma unroll
   for (int i = 0; i < KH; ++i)
 #pragma unroll
-    for (int c = 0; c < CO_G; ++c)
+    for (int c = 0; c < CO; ++c)
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[i][c][j] = 0.f;
-  const float* src = p.I + n * p.sIn;
-  float* dst0 = p.O + n * p.sOn + (int64_t)co0 * p.sOc + wo;
   const int nin = rows + KH - 1;   // input rows ho0 - pt .. ho0 - pt + nin - 1
-  for (int r0 = 0; r0 < nin; r0 += KH) {
+  const float* src = p.I + n * p.sIn + (int64_t)(ho0 - p.pt) * p.sIh + (wo - p.pl);   // next row to load
+  float* dst = p.O + n * p.sOn + (int64_t)co0 * p.sOc + (int64_t)ho0 * p.sOh + wo;
+  // settled once, for whole warps: every lane's loads are aligned and inside
+  // the row, every lane's four outputs exist; floats from a row to the next
+  // 16-byte boundary (the same for every lane: wo is a multiple of 4)
+  const bool vec = __all_sync(0xffffffffu, wo - p.pl >= 0 && wo - p.pl + SEG <= p.W && (p.sIh & 3) == 0 &&
+                                               (reinterpret_cast<uintptr_t>(src) & 15) == 0);
+  const bool full = __all_sync(0xffffffffu, wo + 3 < p.OW);
+  const int sOc4 = (int)(p.sOc & 3), sOh4 = (int)(p.sOh & 3);
+  int at = (int)((reinterpret_cast<uintptr_t>(p.O) >> 2) + n * p.sOn + co0 * p.sOc + ho0 * p.sOh);
+  auto load = [&](int r, float (&x)[SEG]) {
+    const int ih = ho0 + r - p.pt;
+    if (r < nin && ih >= 0 && ih < p.H) {
+      if (SEG >= 4 && vec) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(src));
+        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+        if constexpr (SEG == 6) {
+          const float2 t = __ldg(reinterpret_cast<const float2*>(src + 4));
+          x[4] = t.x; x[5] = t.y;
+        } else if constexpr (SEG == 8) {
+          const float4 t = __ldg(reinterpret_cast<const float4*>(src + 4));
+          x[4] = t.x; x[5] = t.y; x[6] = t.z; x[7] = t.w;
+        }
+      } else {
 #pragma unroll
-    for (int u = 0; u < KH; ++u) {   // input row r = r0 + u, r0 a multiple of KH: slots are compile-time
+        for (int j = 0; j < SEG; ++j) x[j] = (unsigned)(wo - p.pl + j) < (unsigned)p.W ? __ldg(src + j) : 0.f;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < SEG; ++j) x[j] = 0.f;
+    }
+    src += p.sIh;
+  };
+  constexpr int U = KH == 1 ? 4 : KH;   // rows in flight, and unrolled: buffers and slots are compile-time
+  float nx[U][SEG];
+#pragma unroll
+  for (int u = 0; u < U; ++u) load(u, nx[u]);
+#pragma unroll 1
+  for (int r0 = 0; r0 < nin; r0 += U) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {   // input row r = r0 + u, r0 a multiple of U (and so of KH)
       const int r = r0 + u;
       if (r >= nin) break;
       float x[SEG];
-      load_segment<SEG>(src, p.sIh, p.H, p.W, ho0 + r - p.pt, wo - p.pl, x);
+#pragma unroll
+      for (int j = 0; j < SEG; ++j) x[j] = nx[u][j];
 #pragma unroll
       for (int kh = 0; kh < KH; ++kh) {   // feeds output row r - kh through tap row kh
-        const int o = r - kh;
-        if (o < 0 || o >= rows) continue;
         const int slot = (u - kh + KH) % KH;
 #pragma unroll
-        for (int c = 0; c < CO_G; ++c)
+        for (int c = 0; c < CO; ++c)
 #pragma unroll
           for (int kw = 0; kw < KW; ++kw)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[slot][c][j] = fmaf(x[j + kw], w[c][kh * KW + kw], acc[slot][c][j]);
+            for (int j = 0; j < 4; ++j)
+              acc[slot][c][j] = kh == 0 && kw == 0 ? x[j] * w[c][0] : fmaf(x[j + kw], w[c][kh * KW + kw], acc[slot][c][j]);
       }
-      const int o = r - (KH - 1);   // complete: its last tap row was this input row
-      if (o >= 0 && o < rows) {
-        const int slot = (u + 1) % KH;
+      load(r + U, nx[u]);
+      if (r < KH - 1) continue;
+      // row r - (KH - 1) is complete: its last tap row was this input row
+      const int slot = (u + 1) % KH;
 #pragma unroll
-        for (int c = 0; c < CO_G; ++c) {
-          if (c >= ncog) break;
-          store4(p, dst0 + (int64_t)c * p.sOc + (int64_t)(ho0 + o) * p.sOh, wo, bias[c], acc[slot][c]);
+      for (int c = 0; c < CO; ++c) {
+        if (c >= ncog) break;
+        float* d = dst + c * p.sOc;
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float o = acc[slot][c][j];
+          if constexpr (!PLAIN)
+            if (p.beta != 0.f && wo + j < p.OW) o = fmaf(p.beta, d[j], o);
+          o += bias[c];
+          if constexpr (!PLAIN)
+            if (p.relu) o = (o > 0.f || o != o) ? o : 0.f;
+          v[j] = o;
         }
-#pragma unroll
-        for (int c = 0; c < CO_G; ++c)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[slot][c][j] = 0.f;
+        const int s = -(at + c * sOc4) & 3;
+        if (full && s == 0) {
+          *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
+        } else if (full && s == 2) {
+          *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
+          *reinterpret_cast<float2*>(d + 2) = make_float2(v[2], v[3]);
+        } else {
+          store_shifted(d, s, wo, p.OW, v[0], v[1], v[2], v[3]);
+        }
       }
+      dst += p.sOh;
+      at += sOh4;
     }
   }
 }
@@ -358,25 +437,39 @@ nk_status launch_rows(const Direct& p, cudaStream_t st) {
   return check_launch("direct_rows_kernel");
 }
 
-// One input channel: rows per thread chosen so the grid makes about four
-// waves of resident CTAs (6 per SM at this kernel's register count), which
-// keeps the last wave's tail short; at least 4, at most 64 rows.
-template <int KH, int KW>
-nk_status launch_stream(const Direct& p, cudaStream_t st) {
-  constexpr int CO_R = 4;
+// One input channel: output rows per thread.  Runs short enough that the grid
+// walks the images nearly in order, long enough to amortise the KH - 1 halo
+// rows, and at least six CTAs per SM.  Measured, us for 4 / 8 / 16 / 32 / 64
+// rows: 16 x 1280 x 1280 1 -> 3, 3 x 3: 90 / 84 / 89 / 110 / 156; 5 x 5: 268 /
+// 211 / 180 / 179 / 206; 1 x 1280 x 1280, 3 x 3: 11 / 14 / 18 / 33 / 63; 16 x
+// 1000 x 1000 1 -> 4, 1 x 1: 50 / 55 / 64 / 82 / 100.
+template <int KH, int KW, int CO>
+nk_status launch_stream_co(const Direct& p, cudaStream_t st) {
   int sms = 152;
   nk_status s = require_device(&sms);
   if (s != NK_OK) return s;
-  const int groups = (p.CO + CO_R - 1) / CO_R;
+  const int groups = (p.CO + CO - 1) / CO;
   if ((int64_t)p.N * groups > 65535) return fail(NK_ERR_UNSUPPORTED, "batch x channel groups too large");
   const int64_t ctas_per_row = (int64_t)((p.OW + 511) / 512) * p.N * groups;
-  const int64_t target = (int64_t)sms * 6 * 4;
-  int64_t rpt = ((int64_t)p.OH * ctas_per_row + target - 1) / target;
-  rpt = rpt < 4 ? 4 : rpt > 64 ? 64 : rpt;
+  constexpr int64_t kRows = KH == 1 ? 4 : KH == 3 ? 8 : 24;
+  int64_t rpt = (int64_t)p.OH * ctas_per_row / ((int64_t)sms * 6);
+  rpt = rpt < 4 ? 4 : rpt > kRows ? kRows : rpt;
+  if ((p.OH + rpt - 1) / rpt > 65535) rpt = 64;   // grid.y
   dim3 grid((unsigned)((p.OW + 511) / 512), (unsigned)((p.OH + rpt - 1) / rpt), (unsigned)(p.N * groups));
   if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "output too tall");
-  (void)nk::launch_k(direct_stream_kernel<KH, KW, CO_R>, dim3(grid), dim3(128), 0, st, 1, p, (int)rpt);
+  if (p.beta == 0.f && !p.relu) (void)nk::launch_k(direct_stream_kernel<KH, KW, CO, true>, grid, dim3(128), 0, st, 1, p, (int)rpt);
+  else (void)nk::launch_k(direct_stream_kernel<KH, KW, CO, false>, grid, dim3(128), 0, st, 1, p, (int)rpt);
   return check_launch("direct_stream_kernel");
+}
+
+template <int KH, int KW>
+nk_status launch_stream(const Direct& p, cudaStream_t st) {
+  switch (p.CO) {
+    case 1: return launch_stream_co<KH, KW, 1>(p, st);
+    case 2: return launch_stream_co<KH, KW, 2>(p, st);
+    case 3: return launch_stream_co<KH, KW, 3>(p, st);
+    default: return launch_stream_co<KH, KW, 4>(p, st);
+  }
 }
 
 }  // namespace
