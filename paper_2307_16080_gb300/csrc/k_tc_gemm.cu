@@ -63,15 +63,34 @@ int smem_bytes(int kind, int bn, int stages, bool wide = false, int mch = 1) {
 // cluster 1 are tall tiles of 2 / 4 chains (tile_m 256 with cluster 2 is a pair).
 int chains_of(const nk_schedule& s) { return (s.cluster == 1 && s.tile_m > 128) ? s.tile_m / 128 : 1; }
 
+// Wide tiles: 512 columns, or 256 of BF16x3 (two accumulators), fill the TMEM.
+bool is_wide(int kind, const nk_schedule& s) { return s.tile_n == 512 || (kind == TC_BF16X3 && s.tile_n == 256); }
+
+// BF16x3 with no schedule given: 256 x 256 tiles on CTA pairs where they win.
+// A 128 x 128 tile loads 64 KB for 768 cycles of MMAs, more than L2 delivers;
+// a CTA of the wide pair loads 64 KB for 1536, but its accumulators have no
+// second buffer, so every tile's epilogue is exposed.  Microseconds of a wave,
+// fitted: 0.62 per 64-deep K block + 1.5 (128 x 128), 1.0 + 6 (wide).  Whole
+// calls, 128 x 128 against wide: 4096^3 329 / 311 us, 4096 x 4096 x 1024 92 /
+// 96, 1024 x 4096 x 1024 33.0 / 32.2, 3001 x 2002 x 1999 87 / 99.  The schedule
+// space has no such point: a caller's schedule is always taken as it is.
+bool x3_wide_wins(int M, int N, int K, int sms) {
+  const int64_t wide = (int64_t)((M + 255) / 256) * ((N + 255) / 256);
+  const int64_t square = (int64_t)((M + 127) / 128) * ((N + 127) / 128);
+  const int64_t pairs = sms / 2;
+  const double nkb = (K + 63) / 64;
+  return (wide + pairs - 1) / pairs * (1.0 * nkb + 6.0) < (square + sms - 1) / sms * (0.62 * nkb + 1.5);
+}
+
 // Shared memory of a schedule: a CTA of a pair (tile_m 256) keeps half of B.
 int smem_of(int kind, const nk_schedule& s) {
   const bool pair = s.cluster == 2 && s.tile_m == 256;
-  return smem_bytes(kind, pair ? s.tile_n / 2 : s.tile_n, s.stages, s.tile_n == 512, chains_of(s));
+  return smem_bytes(kind, pair ? s.tile_n / 2 : s.tile_n, s.stages, is_wide(kind, s), chains_of(s));
 }
 
 // CTAs that fit on one SM: shared memory and the 512 TMEM columns.
 int ctas_per_sm(int kind, const nk_schedule& s) {
-  if (s.tile_n == 512) return 1;   // a wide tile holds all 512 TMEM columns
+  if (is_wide(kind, s)) return 1;   // a wide tile holds all 512 TMEM columns
   const int bn = s.tile_n;
   const int sm = smem_of(kind, s);
   int by_smem = kMaxSmem / sm;
@@ -132,13 +151,16 @@ size_t tc_gemm_ws(const TcGemm& g, const nk_schedule& s) {
   return (size_t)s.split_k * g.M * g.N * sizeof(float);
 }
 
-nk_status tc_gemm(const TcGemm& g, const nk_schedule& s, void* ws, size_t ws_bytes, cudaStream_t st) {
+nk_status tc_gemm(const TcGemm& g, const nk_schedule& sched, void* ws, size_t ws_bytes, cudaStream_t st) {
+  nk_schedule s = sched;
   int sms = 0;
   nk_status status = require_device(&sms);
   if (status != NK_OK) return status;
   if (g.M <= 0 || g.N <= 0) return NK_OK;
   if (!tc_schedule_valid(g.kind, s, g.M, g.N, g.K))
     return fail(NK_ERR_NO_SCHEDULE, "illegal tensor-core schedule");
+  if (g.any_schedule && g.kind == TC_BF16X3 && s.split_k == 1 && x3_wide_wins(g.M, g.N, g.K, sms))
+    s = nk_schedule{256, 256, 64, 2, 3, 1};
   if (g.K <= 0) {
     // Empty reduction: the epilogue alone (the CUDA-core kernel with K = 0).
     SimtGemm z{};
@@ -199,26 +221,28 @@ nk_status tc_gemm(const TcGemm& g, const nk_schedule& s, void* ws, size_t ws_byt
                     (splits == 1 || (g.N % 4 == 0 && (reinterpret_cast<uintptr_t>(ws) & 15) == 0));
   p.c_vec = cvec ? 1 : 0;
   p.c_vec32 = (splits == 1 && (reinterpret_cast<uintptr_t>(g.C) & 31) == 0 && g.ldc % 8 == 0) ? 1 : 0;
-  // TMA-store epilogue: plain overwrite of a 16-byte aligned C in one K slice.
-  // Rows must also end on a 16-byte boundary (N % 4 == 0): a TMA store clips
-  // the innermost dimension only to 16-byte granules, so with N % 4 != 0 and
-  // a padded row stride it wrote the row's padding (caught by canaries).
+  // Staged epilogue: plain overwrite of C in one K slice, by TMA stores where C
+  // is 16-byte aligned.  Rows must also end on a 16-byte boundary (N % 4 == 0):
+  // a TMA store clips the innermost dimension only to 16-byte granules, so
+  // with N % 4 != 0 and a padded row stride it wrote the row's padding (caught
+  // by canaries).  Any other C is copied out by the warps.
   p.c_tma = 0;
-  if (mch == 1 && splits == 1 && g.beta == 0.f && (g.ew.n == 0 || g.kind != TC_BF16X3) && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0 &&
-      (g.ldc * 4) % 16 == 0 && g.N % 4 == 0) {
+  if (mch == 1 && splits == 1 && g.beta == 0.f && (g.ew.n == 0 || g.kind != TC_BF16X3)) {
+    p.c_tma = 2;
     auto fn = encode_fn();
     cuuint64_t dims[2] = {(cuuint64_t)g.N, (cuuint64_t)g.M};
     cuuint64_t strides[1] = {(cuuint64_t)(g.ldc * 4)};
     cuuint32_t box[2] = {32, 32};
     cuuint32_t es[2] = {1, 1};
-    if (fn && fn(&p.tmC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, es,
-                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+    if ((reinterpret_cast<uintptr_t>(g.C) & 15) == 0 && (g.ldc * 4) % 16 == 0 && g.N % 4 == 0 && fn &&
+        fn(&p.tmC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
       p.c_tma = 1;
   }
   int smem = smem_of(g.kind, s);
   const int per_sm = ctas_per_sm(g.kind, s);
-  const bool wide = s.tile_n == 512;
+  const bool wide = is_wide(g.kind, s);
   // Eight epilogue warps when a CTA has the SM to itself, and a second staging
   // box per warp where shared memory has room beside the SM's CTAs.
   const bool ep8 = p.c_tma && !wide && per_sm == 1 && smem + 4 * kStageBox <= kMaxSmem;

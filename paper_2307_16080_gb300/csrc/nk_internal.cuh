@@ -212,6 +212,7 @@ struct TcGemm {
   const float* scale_a;   // device scalars (FP8 computed on device) or null
   const float* scale_b;
   EwProg ew;              // epilogue program (offsets from C)
+  bool any_schedule;      // the caller gave no schedule: tc_gemm may take a better one of its own
 };
 
 nk_status tc_gemm(const TcGemm& g, const nk_schedule& s, void* ws, size_t ws_bytes,

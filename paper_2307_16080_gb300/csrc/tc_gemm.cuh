@@ -19,8 +19,8 @@
 //               alpha, beta*C, bias, ReLU and stores -- overlapping the
 //               next tile's main loop through the second accumulator.
 //
-// BF16x3 issues three MMAs per K step (hi*hi, hi*lo, lo*hi) into the same
-// accumulator.  Split-K writes each slice's raw tile to the workspace and the
+// BF16x3 sums hi*hi, hi*lo and lo*hi per K step: on one CTA in two MMAs, hi *
+// [hi lo] over two adjacent accumulators and lo * hi into the second.  Split-K writes each slice's raw tile to the workspace and the
 // fixed-order warp-shuffle reduce applies the epilogue.
 //
 // Every wait is bounded (see tc_ptx.cuh); on a timeout the CTA drains its own
@@ -75,7 +75,7 @@ struct TcParams {
   uint32_t a_box_bytes;         // bytes TMA writes per A stage (16 KB unless a conv tile is short)
   // epilogue through shared memory and TMA stores (plain GEMM, beta = 0, one K slice)
   CUtensorMap tmC;
-  int c_tma;
+  int c_tma;                    // 1: TMA stores; 2: C has no tensor map, the warp copies the box out
   int boxes2;                   // c_tma: two staging boxes per epilogue warp
   EwProg ew;                    // fused elementwise program (offsets from C), single launches
   int out_bf16;                 // single convolutions: C holds BF16 (RNE of the FP32 result)
@@ -247,6 +247,9 @@ __device__ __forceinline__ int conv_row(const ConvTile& c, int tm, int r) {
 // that latency.  Both chains fill the 512 TMEM columns, so the accumulator is
 // single-buffered and eight epilogue warps drain it.
 //
+// For BF16x3 a wide tile is 256 x 256: its two N = 256 accumulators are hi*hi
+// and the corrections.
+//
 // MCH > 1 (tall tile, one CTA): MCH stacked 128-row tiles of A share one B
 // tile, each with its own accumulator chain, so narrow problems (N = 64, 128)
 // keep several independent MMA chains in flight.
@@ -274,7 +277,7 @@ template <int KIND, int CL, bool GROUPED, bool CONV = false, bool PAIR = false, 
 __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIND == TC_BF16X3) ? 1 : 2) tc_gemm_kernel(const __grid_constant__ TcParams p) {
   static_assert(!EP8 || (!WIDE && MCH == 1 && !CONV), "eight epilogue warps: plain GEMM tiles");
   static_assert(PAIR == (CL == 2), "a cluster of two is a CTA pair, and a CTA pair is a cluster of two");
-  static_assert(!WIDE || (PAIR && KIND != TC_BF16X3 && !GROUPED), "wide tiles are pair tiles");
+  static_assert(!WIDE || (PAIR && !GROUPED), "wide tiles are pair tiles");
   static_assert(MCH == 1 || (!PAIR && !GROUPED && KIND != TC_BF16X3 && CL == 1), "tall tiles: one CTA");
   static_assert(!EW || (!GROUPED && !CONV && MCH == 1), "programs in registers: single GEMMs with TMA stores");
   extern __shared__ uint8_t smem_raw[];
@@ -360,9 +363,14 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
 
   const int a_bytes = MCH * kBM * kRowBytes;
   const int b_bytes = b_rows_smem * kRowBytes;
-  // Stage layout: [A][B] or, for BF16x3, [A_hi][B_hi][A_lo][B_lo].
-  auto a_smem = [&](int s, int part) { return base + s * sb + part * (a_bytes + b_bytes); };
-  auto b_smem = [&](int s, int part) { return base + s * sb + part * (a_bytes + b_bytes) + a_bytes; };
+  // Stage layout: [A][B] or, for BF16x3, [A_hi][A_lo][B_hi][B_lo] on one CTA
+  // (B_hi and B_lo adjacent: one B operand of 2 * bn rows), and
+  // [A_hi][B_hi][A_lo][B_lo] on a pair.
+  constexpr bool HILO = KIND == TC_BF16X3 && !PAIR;
+  auto a_smem = [&](int s, int part) { return base + s * sb + part * (HILO ? a_bytes : a_bytes + b_bytes); };
+  auto b_smem = [&](int s, int part) {
+    return base + s * sb + (HILO ? 2 * a_bytes + part * b_bytes : part * (a_bytes + b_bytes) + a_bytes);
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
@@ -395,7 +403,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
             } else {
               if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(s), 2u * (uint32_t)sb);
               const int kx = kb * kblk;
-              if (WIDE) {
+              if (WIDE && KIND != TC_BF16X3) {
                 // chain h (N columns h*256 .. h*256+255): this CTA holds its 128 rows of B^T
                 ptx::tma_load_2d_pair(a_smem(s, 0), t.ma, lf, kx, t.tm * kBM);
                 ptx::tma_load_2d_pair(b_smem(s, 0), t.mb, lf, kx, t.tn * p.bn + rank * 128);
@@ -456,6 +464,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
     // -------------------------------------------------------------- MMA
     if (lane == 0 && (!PAIR || rank == 0)) {
       const uint32_t idesc = ptx::make_idesc(KIND == TC_FP8 ? 0 : 1, PAIR ? 2 * kBM : kBM, WIDE ? 256 : p.bn);
+      const uint32_t idesc2 = HILO ? ptx::make_idesc(1, kBM, 2 * p.bn) : 0u;
       int it = 0, tc = 0;
       bool ok = true;
       for (int u = cluster_id; u < p.units && ok; u += n_clusters, ++tc) {
@@ -479,6 +488,15 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
             const uint64_t ad = ptx::sw128_desc(a_smem(s, 0) + koff);
             const uint64_t bd = ptx::sw128_desc(b_smem(s, 0) + koff);
             const uint32_t accum = (kb > kb0 || k > 0) ? 1u : 0u;
+            if constexpr (HILO) {
+              // hi * [hi lo] in one MMA over both accumulators, then lo * hi.
+              // An MMA of this kernel takes about as long at N = 128 as at
+              // 256, so two a step instead of three: 4096^3, with its casts,
+              // 364 -> 329 us (L2 now bounds it: see x3_wide_wins).
+              ptx::tc_mma<0>(d, ad, bd, idesc2, accum);
+              ptx::tc_mma<0>(d2, ptx::sw128_desc(a_smem(s, 1) + koff), bd, idesc, 1u);
+              continue;
+            }
             if (PAIR) ptx::tc_mma_pair<KIND == TC_FP8>(d, ad, bd, idesc, accum);
             else ptx::tc_mma<KIND == TC_FP8>(d, ad, bd, idesc, accum);
 #pragma unroll
@@ -486,20 +504,15 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
               ptx::tc_mma<KIND == TC_FP8>(d + (uint32_t)(ch * p.bn),
                                           ptx::sw128_desc(a_smem(s, 0) + ch * kBM * kRowBytes + koff), bd, idesc,
                                           accum);
-            if (WIDE) {   // second chain: B^T rows 128..255 of this CTA's stage
+            if (WIDE && KIND != TC_BF16X3) {   // second chain: B^T rows 128..255 of this CTA's stage
               const uint64_t bw = ptx::sw128_desc(b_smem(s, 0) + 128 * kRowBytes + koff);
               ptx::tc_mma_pair<KIND == TC_FP8>(d2, ad, bw, idesc, accum);
             }
-            if (KIND == TC_BF16X3) {
+            if constexpr (KIND == TC_BF16X3 && PAIR) {
               const uint64_t ad2 = ptx::sw128_desc(a_smem(s, 1) + koff);
               const uint64_t bd2 = ptx::sw128_desc(b_smem(s, 1) + koff);
-              if (PAIR) {
-                ptx::tc_mma_pair<0>(d2, ad, bd2, idesc, accum);   // hi * lo
-                ptx::tc_mma_pair<0>(d2, ad2, bd, idesc, 1u);      // lo * hi
-              } else {
-                ptx::tc_mma<0>(d2, ad, bd2, idesc, accum);   // hi * lo
-                ptx::tc_mma<0>(d2, ad2, bd, idesc, 1u);      // lo * hi
-              }
+              ptx::tc_mma_pair<0>(d2, ad, bd2, idesc, accum);   // hi * lo
+              ptx::tc_mma_pair<0>(d2, ad2, bd, idesc, 1u);      // lo * hi
             }
           }
           if (PAIR) ptx::tc_commit_pair_mc(empty_bar(s), (uint16_t)0x3);
@@ -551,8 +564,8 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
           // 37.0 and 89.4 -> 35.5 us; 8192^3 609 -> 560 us; FP8 4096^3 79 -> 53 us.
           const int row = t.tm * kBM + q * 32 + lane;
           const bool row_ok = row < t.M;
-          const int c_begin = WIDE ? ((warp - 2) / 4) * 256 : EP8 ? ((warp - 2) / 4) * (p.bn / 2) : 0;
-          const int c_cols = WIDE ? 256 : EP8 ? p.bn / 2 : p.bn;
+          const int c_cols = (WIDE || EP8) ? p.bn / 2 : p.bn;   // eight warps: two per lane quarter, half the columns each
+          const int c_begin = (WIDE || EP8) ? ((warp - 2) / 4) * c_cols : 0;
           const int col_begin = t.tn * p.bn + c_begin;
           const int nseg = max(0, min(c_cols, t.N - col_begin) + 31) / 32;
           const uint32_t ta0 = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * acc_cols + c_begin);
@@ -609,6 +622,28 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
                            "f"(v[4 * j16 + 2]), "f"(v[4 * j16 + 3])
                            : "memory");
             }
+            if (p.c_tma == 2) {
+              // rows of C that no TMA store can address (N or the row stride
+              // not a multiple of 4, or a C off 16 bytes): the warp writes the
+              // box row by row, 128 contiguous bytes each, where a lane per
+              // row touched 32 sectors with every store: BF16x3 3001
+              // x 2002 x 1999, whole call, 104 -> 87 us.
+              __syncwarp();
+              const int rows = min(32, t.M - (t.tm * kBM + q * 32));
+              float* dst = t.C + (int64_t)(t.tm * kBM + q * 32) * t.ldc + col0 + lane;
+              const bool in = col0 + lane < t.N;
+#pragma unroll 8
+              for (int r = 0; r < rows; ++r) {
+                float x;
+                asm volatile("ld.shared.f32 %0, [%1];"
+                             : "=f"(x)
+                             : "r"(stg + (uint32_t)(r * 128 + (((lane >> 2) ^ (r & 7)) * 16) + (lane & 3) * 4))
+                             : "memory");
+                if (in) dst[(int64_t)r * t.ldc] = x;
+              }
+              __syncwarp();
+              return;
+            }
             ptx::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
@@ -640,8 +675,8 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
       const int row = CONV ? conv_row(*t.cv, tmc, q * 32 + lane) : tmc * kBM + q * 32 + lane;
       const bool row_ok = CONV ? row >= 0 : row < t.M;
       // a wide tile has two warps per lane quarter, each draining one chain's 256 columns
-      const int c_begin = WIDE ? ((warp - 2) / 4) * 256 : EP8 ? ((warp - 2) / 4) * (p.bn / 2) : 0;
-      const int c_end = WIDE ? c_begin + 256 : EP8 ? c_begin + p.bn / 2 : p.bn;
+      const int c_begin = (WIDE || EP8) ? ((warp - 2) / 4) * (p.bn / 2) : 0;
+      const int c_end = (WIDE || EP8) ? c_begin + p.bn / 2 : p.bn;
       for (int c0 = c_begin; c0 < c_end; c0 += 32) {
         float v[32];
         const uint32_t ta =
@@ -835,6 +870,10 @@ nk_status launch(const TcParams& p, int grid, int smem, cudaStream_t st) {
 template <bool EW, bool EP8>
 nk_status launch_single(const TcParams& p, const nk_schedule& s, int kind, int mch, int grid, int smem,
                         cudaStream_t st) {
+  if constexpr (!EP8 && !EW) {
+    if (kind == TC_BF16X3 && s.tile_n == 256)
+      return launch<TC_BF16X3, 2, false, false, true, true>(p, grid, smem, st);
+  }
   if constexpr (!EP8) {
     if (s.tile_n == 512) {
       if (kind == TC_FP8) return launch<TC_FP8, 2, false, false, true, true, 1, false, EW>(p, grid, smem, st);

@@ -106,3 +106,35 @@ def test_steps_over_the_range_of_fp32(nk, name):
     assert np.isnan(got[np.isnan(v)]).all()
     if name != "sigmoid":
         assert np.array_equal(np.signbit(got[v == 0]), np.signbit(v[v == 0]))
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp8", "bf16x3"])
+@pytest.mark.parametrize("M,N,K,ldc", [(1, 1, 8, 1), (33, 31, 40, 31), (300, 770, 136, 771), (257, 515, 64, 519),
+                                       (129, 36, 300, 37)])
+def test_outputs_without_a_tensor_map(nk, prec, M, N, K, ldc):
+    """C whose rows no TMA store can address is copied out by the warps: odd N,
+    odd row strides, every tile, with a bias and a program."""
+    A, B = synth.small_ints(904, 0, (M, K), -7, 7) / 2, synth.small_ints(904, 1, (K, N), -7, 7) / 2
+    A[0, 0] = B[0, 0] = 3.5
+    bias = synth.small_ints(904, 2, (N,))
+    want = A.astype(np.float64) @ B + bias
+    for sched in [None] + TILES[prec]:
+        for ew in (None, [("affine", 0.5, 1.0), ("relu",)]):
+            C = Canary((M, N), strides=(ldc, 1), pad=4097)
+            nk.nk_matmul(dev(A), dev(B), C.t, prec, bias=dev(bias), schedule=sched, ew=ew)
+            nk.nk_sync_status()
+            assert np.array_equal(host(C.t), (want if ew is None else np.maximum(want * 0.5 + 1, 0)).astype(np.float32))
+            C.check()
+
+
+@pytest.mark.parametrize("M,N,K", [(4096, 4096, 4096), (3841, 4100, 4000), (1024, 4097, 1024)])
+def test_bf16x3_wide_pairs(nk, M, N, K):
+    """No schedule given: the sizes where BF16x3 takes its 256 x 256 pair tiles
+    give the bits of the 128 x 128 ones (the same products in the same order)."""
+    g = torch.Generator(device=DEV).manual_seed(5)
+    A, B = torch.randn(M, K, generator=g, device=DEV), torch.randn(K, N, generator=g, device=DEV)
+    C, R = torch.empty(M, N, device=DEV), torch.empty(M, N, device=DEV)
+    nk.nk_matmul(A, B, C, "bf16x3")
+    nk.nk_matmul(A, B, R, "bf16x3", schedule=(128, 128, 64, 1, 3, 1))
+    nk.nk_sync_status()
+    assert torch.equal(C, R)
