@@ -459,19 +459,23 @@ nk_status nk_matmul(const nk_tensor* A, const nk_tensor* B, nk_tensor* C, int32_
   void* a1 = kind == TC_BF16X3 ? w + P.off_a2 : nullptr;
   void* b1 = kind == TC_BF16X3 ? w + P.off_b2 : nullptr;
   const int ck = kind == TC_BF16 ? 0 : kind == TC_FP8 ? 1 : 2;
+  // Each operand's amax directly before its own cast, which then finds what it
+  // reads in L2 (both amaxes first, and A is gone when its cast begins).
+  void* aw = w + P.off_amax;
+  const size_t awb = prep_amax_ws(0);
   if (kind == TC_FP8) {
-    void* aw = w + P.off_amax;
-    const size_t awb = prep_amax_ws(0);
     if (a_kmajor) s = prep_amax(Af, P.M, P.K, P.A.s0, scal + 0, aw, awb, st, &pro_a);
     else s = prep_amax(Af, P.K, P.M, P.A.s1, scal + 0, aw, awb, st, &pro_a);
-    if (s != NK_OK) return s;
-    if (b_kmajor) s = prep_amax(Bf, P.N, P.K, P.B.s1, scal + 1, aw, awb, st, &pro_b);
-    else s = prep_amax(Bf, P.K, P.N, P.B.s0, scal + 1, aw, awb, st, &pro_b);
     if (s != NK_OK) return s;
   }
   if (a_kmajor) s = prep_cast(ck, Af, P.M, P.K, P.A.s0, scal + 0, a0, a1, P.ldk, 0, scal + 2, st, &pro_a);
   else s = prep_cast(ck, Af, P.K, P.M, P.A.s1, scal + 0, a0, a1, P.ldk, 1, scal + 2, st, &pro_a);
   if (s != NK_OK) return s;
+  if (kind == TC_FP8) {
+    if (b_kmajor) s = prep_amax(Bf, P.N, P.K, P.B.s1, scal + 1, aw, awb, st, &pro_b);
+    else s = prep_amax(Bf, P.K, P.N, P.B.s0, scal + 1, aw, awb, st, &pro_b);
+    if (s != NK_OK) return s;
+  }
   if (b_kmajor) s = prep_cast(ck, Bf, P.N, P.K, P.B.s1, scal + 1, b0, b1, P.ldk, 0, scal + 3, st, &pro_b);
   else s = prep_cast(ck, Bf, P.K, P.N, P.B.s0, scal + 1, b0, b1, P.ldk, 1, scal + 3, st, &pro_b);
   if (s != NK_OK) return s;
