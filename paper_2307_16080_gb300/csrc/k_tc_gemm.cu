@@ -88,24 +88,6 @@ int smem_of(int kind, const nk_schedule& s) {
   return smem_bytes(kind, pair ? s.tile_n / 2 : s.tile_n, s.stages, is_wide(kind, s), chains_of(s));
 }
 
-// Whether a product's K slices are summed inside a cluster (2, 4 or 8 slices,
-// one 128-row tile per CTA, room for the partial tile over the stages) instead
-// of by a reduce pass over the workspace; both add in the same order.  The
-// cluster's launch and exchange cost about 3 us, so slices of a few K blocks
-// stay with the reduce pass.  Cluster / reduce, us: BF16 512 x 512 x 4096 (4
-// slices of 16 blocks) 11.6 / 16.9, 1907 x 133 x 5000 (2 of 40) 20.7 / 29.5, 256
-// x 256 x 2048 (8 of 4) 7.3 / 10.1; BF16x3 512 x 512 x 2048 (8 of 4) 25.1 /
-// 23.5.  Convolutions keep the reduce pass: repeated alone they gain as much
-// (8x14x14x256 -> 512 3x3 / 2: 11.5 / 15.0), but between other layers the
-// exchange's code comes from L2 each time, and a 20-layer forward at batch 8
-// lost 7 us.
-bool sums_in_cluster(int kind, const nk_schedule& s, int splits, int kb_per_split, int64_t units, int sms) {
-  if (splits != s.split_k || (splits != 2 && splits != 4 && splits != 8)) return false;
-  if (s.cluster != 1 || chains_of(s) != 1 || s.tile_m != 128) return false;
-  if (kb_per_split < 8 && (splits < 4 || kind == TC_BF16X3)) return false;
-  return s.stages * stage_bytes(kind, s.tile_n) >= partial_bytes(s.tile_n) && units <= 4 * (int64_t)sms;
-}
-
 // CTAs that fit on one SM: shared memory and the 512 TMEM columns.
 int ctas_per_sm(int kind, const nk_schedule& s) {
   if (is_wide(kind, s)) return 1;   // a wide tile holds all 512 TMEM columns
@@ -263,7 +245,6 @@ nk_status tc_gemm(const TcGemm& g, const nk_schedule& sched, void* ws, size_t ws
   const bool wide = is_wide(g.kind, s);
   // Eight epilogue warps when a CTA has the SM to itself, and a second staging
   // box per warp where shared memory has room beside the SM's CTAs.
-  if (splits > 1 && sums_in_cluster(g.kind, s, splits, p.kb_per_split, p.units, sms)) p.csplit = splits;
   const bool ep8 = p.c_tma && !wide && per_sm == 1 && smem + 4 * kStageBox <= kMaxSmem;
   if (ep8) smem += 4 * kStageBox;
   p.boxes2 = p.c_tma && per_sm * (smem + staging_bytes(wide || ep8)) <= kMaxSmem ? 1 : 0;
@@ -271,12 +252,12 @@ nk_status tc_gemm(const TcGemm& g, const nk_schedule& sched, void* ws, size_t ws
   int grid = sms * per_sm;
   grid = grid / CL * CL;
   const int need_ctas = p.units * CL;
-  if (grid > need_ctas || p.csplit) grid = need_ctas;
+  if (grid > need_ctas) grid = need_ctas;
   if (grid < CL) grid = CL;
   if (p.ew.n && p.c_tma) status = tc_gemm_ew_launch(p, s, g.kind, ep8, grid, smem, st);
   else if (ep8) status = launch_single<false, true>(p, s, g.kind, mch, grid, smem, st);
   else status = launch_single<false, false>(p, s, g.kind, mch, grid, smem, st);
-  if (status != NK_OK || splits == 1 || p.csplit) return status;
+  if (status != NK_OK || splits == 1) return status;
   SplitReduce r{};
   r.partial = p.partial;
   r.splits = splits;

@@ -30,7 +30,6 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
-#include "cluster_sum.cuh"
 #include "nk_internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -57,7 +56,6 @@ struct TcParams {
   float* C;
   int64_t ldc;
   float* partial;         // [splits][M][N] when splits > 1
-  int csplit;             // splits summed inside a cluster of as many CTAs (0: not)
   const float* bias;
   int bias_on_m, relu;
   float beta, alpha;
@@ -315,11 +313,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
   const int warp = threadIdx.x / 32;
   const int lane = threadIdx.x % 32;
   const int rank = CL == 2 ? (int)ptx::cluster_ctarank() : 0;
-  // K slices in a cluster (csplit): every CTA has one unit, and the CTAs of a
-  // cluster the slices of one tile.
-  constexpr bool CSPLIT = CL == 1 && !GROUPED && !CONV && MCH == 1 && !EP8 && !EW;
-  const int cs = CSPLIT ? p.csplit : 0;
-  const int cluster_id = cs > 1 ? (int)(blockIdx.x % cs) * (p.units / cs) + (int)(blockIdx.x / cs) : (int)blockIdx.x / CL;
+  const int cluster_id = blockIdx.x / CL;
   const int n_clusters = gridDim.x / CL;
   // Accumulator columns per buffer: BN, or 2*BN for BF16x3 (hi*hi and the
   // hi*lo + lo*hi corrections accumulate apart and meet in the epilogue, so
@@ -695,12 +689,6 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
           for (int j = 0; j < 32; ++j) v[j] += w[j];
         }
         const int col0 = t.tn * p.bn + c0;
-        if constexpr (CSPLIT) {
-          if (cs > 1) {
-            store_partial32(base, p.bn, q * 32 + lane, c0, v);
-            continue;
-          }
-        }
         if (!row_ok || col0 >= t.N) continue;
         if (p.partial) {
           float* dst = p.partial + ((int64_t)t.split * p.M + row) * p.N + col0;
@@ -856,23 +844,6 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
     else ptx::tmem_dealloc(tmem_base, tmem_cols);
   }
   if (CL == 2) ptx::cluster_sync();
-  if constexpr (CSPLIT) {
-    if (cs > 1) {
-      // All copies and MMAs of this CTA are done and its partial tile lies over
-      // the pipeline stages; every CTA takes 128 / cs rows of the tile.
-      ptx::cluster_sync();
-      const UnitView t = view_unit<GROUPED>(p, cluster_id, CL, rank);
-      RowOut o{t.C, t.N, t.bias, p.bias_on_m, t.relu, p.alpha, t.beta};
-      if (p.scale_a) o.alpha = __frcp_rn(__fmul_rn(*p.scale_a, *p.scale_b));
-      finish_tile<kThreads>(o, p.ew, base, p.bn, cs, (int)ptx::cluster_ctarank(), t.tn * p.bn,
-                            [&](int r, int64_t& off, int& m) {
-                              m = t.tm * kBM + r;
-                              off = (int64_t)m * t.ldc;
-                              return m < t.M;
-                            });
-      ptx::cluster_sync();   // no CTA leaves while another may still read its tile
-    }
-  }
 }
 
 template <int KIND, int CL, bool GROUPED = false, bool CONV = false, bool PAIR = false, bool WIDE = false,
@@ -888,8 +859,7 @@ nk_status launch(const TcParams& p, int grid, int smem, cudaStream_t st) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(tc_gemm_kernel)");
     if (dev >= 0 && dev < 64) set_bytes[dev] = smem;
   }
-  const cudaError_t e = nk::launch_k(kern, dim3(grid), dim3((WIDE || EP8) ? 320 : kThreads), smem, st,
-                                   p.csplit > 1 ? p.csplit : CL, p);
+  const cudaError_t e = nk::launch_k(kern, dim3(grid), dim3((WIDE || EP8) ? 320 : kThreads), smem, st, CL, p);
   if (e != cudaSuccess) return cuda_fail(e, "launch tc_gemm_kernel");
   return check_launch("tc_gemm_kernel");
 }
