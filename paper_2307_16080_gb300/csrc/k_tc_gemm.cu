@@ -146,9 +146,13 @@ nk_schedule tc_default_schedule(int kind, int M, int N, int K, int sms) {
   return s;
 }
 
+// Split-K partials: rows of N rounded up to 16 bytes, so that every row takes
+// 16-byte stores and loads.
+static int partial_ld(int N) { return (N + 3) / 4 * 4; }
+
 size_t tc_gemm_ws(const TcGemm& g, const nk_schedule& s) {
   if (s.split_k <= 1) return 0;
-  return (size_t)s.split_k * g.M * g.N * sizeof(float);
+  return (size_t)s.split_k * g.M * partial_ld(g.N) * sizeof(float);
 }
 
 nk_status tc_gemm(const TcGemm& g, const nk_schedule& sched, void* ws, size_t ws_bytes, cudaStream_t st) {
@@ -204,9 +208,11 @@ nk_status tc_gemm(const TcGemm& g, const nk_schedule& sched, void* ws, size_t ws
   p.ldc = g.ldc;
   p.partial = nullptr;
   if (splits > 1) {
-    const size_t need = (size_t)splits * g.M * g.N * sizeof(float);
+    const size_t need = (size_t)splits * g.M * partial_ld(g.N) * sizeof(float);
     if (!ws || ws_bytes < need) return fail(NK_ERR_WORKSPACE, "split-K needs %zu bytes of workspace", need);
     p.partial = static_cast<float*>(ws);
+    p.ldp = partial_ld(g.N);
+    p.part_vec = (reinterpret_cast<uintptr_t>(ws) & 15) == 0;
   }
   p.bias = g.bias;
   p.bias_on_m = g.bias_on_m;
@@ -217,8 +223,7 @@ nk_status tc_gemm(const TcGemm& g, const nk_schedule& sched, void* ws, size_t ws
   p.scale_b = g.scale_b;
   p.ew = g.ew;
   p.budget = wait_budget();
-  const bool cvec = ((reinterpret_cast<uintptr_t>(g.C) & 15) == 0) && (g.ldc % 4 == 0) &&
-                    (splits == 1 || (g.N % 4 == 0 && (reinterpret_cast<uintptr_t>(ws) & 15) == 0));
+  const bool cvec = ((reinterpret_cast<uintptr_t>(g.C) & 15) == 0) && (g.ldc % 4 == 0);
   p.c_vec = cvec ? 1 : 0;
   p.c_vec32 = (splits == 1 && (reinterpret_cast<uintptr_t>(g.C) & 31) == 0 && g.ldc % 8 == 0) ? 1 : 0;
   // Staged epilogue: plain overwrite of C in one K slice, by TMA stores where C
@@ -260,6 +265,7 @@ nk_status tc_gemm(const TcGemm& g, const nk_schedule& sched, void* ws, size_t ws
   if (status != NK_OK || splits == 1) return status;
   SplitReduce r{};
   r.partial = p.partial;
+  r.ldp = p.ldp;
   r.splits = splits;
   r.M = g.M;
   r.N = g.N;
@@ -413,7 +419,7 @@ nk_schedule tc_conv_default_schedule(const ConvGeom& g, int F, int sms, int kind
 
 size_t tc_conv_ws(const TcConv& c, const nk_schedule& s) {
   if (s.split_k <= 1 || halo_schedule(c.g, s, c.kind)) return 0;
-  return (size_t)s.split_k * c.g.n * c.g.oh * c.g.ow * c.F * sizeof(float);
+  return (size_t)s.split_k * c.g.n * c.g.oh * c.g.ow * partial_ld(c.F) * sizeof(float);
 }
 
 nk_status tc_conv(const TcConv& c, const nk_schedule& s, void* ws, size_t ws_bytes, cudaStream_t st) {
@@ -455,9 +461,11 @@ nk_status tc_conv(const TcConv& c, const nk_schedule& s, void* ws, size_t ws_byt
   p.C = c.O;
   p.ldc = c.F;
   if (splits > 1) {
-    const size_t need = (size_t)splits * M * c.F * sizeof(float);
+    const size_t need = (size_t)splits * M * partial_ld(c.F) * sizeof(float);
     if (!ws || ws_bytes < need) return fail(NK_ERR_WORKSPACE, "split-K needs %zu bytes of workspace", need);
     p.partial = static_cast<float*>(ws);
+    p.ldp = partial_ld(c.F);
+    p.part_vec = (reinterpret_cast<uintptr_t>(ws) & 15) == 0;
   }
   p.bias = c.bias;
   p.relu = c.relu;
@@ -472,9 +480,8 @@ nk_status tc_conv(const TcConv& c, const nk_schedule& s, void* ws, size_t ws_byt
   p.c_vec32 = (splits == 1 && (reinterpret_cast<uintptr_t>(c.O) & 31) == 0 && c.F % (c.out_bf16 ? 16 : 8) == 0) ? 1 : 0;
   p.resid = (c.ew.n == 2 && c.ew.op[0] == NK_EW_ADD && c.ew.op[1] == NK_EW_RELU &&
              (reinterpret_cast<uintptr_t>(c.ew.t[0]) & 31) == 0 && c.F % 8 == 0) ? 1 : 0;
-  // vector stores: 16-byte aligned rows (FP32: F % 4, BF16: F % 8) and partials
-  p.c_vec = ((reinterpret_cast<uintptr_t>(c.O) & 15) == 0 && c.F % (c.out_bf16 ? 8 : 4) == 0 &&
-             (splits == 1 || (reinterpret_cast<uintptr_t>(ws) & 15) == 0)) ? 1 : 0;
+  // vector stores: 16-byte aligned rows (FP32: F % 4, BF16: F % 8)
+  p.c_vec = ((reinterpret_cast<uintptr_t>(c.O) & 15) == 0 && c.F % (c.out_bf16 ? 8 : 4) == 0) ? 1 : 0;
   const int smem = smem_of(kind, s);
   if (smem > kMaxSmem) return fail(NK_ERR_NO_SCHEDULE, "conv schedule needs %d bytes of shared memory", smem);
   int grid = sms * ctas_per_sm(kind, s);
@@ -492,6 +499,7 @@ nk_status tc_conv(const TcConv& c, const nk_schedule& s, void* ws, size_t ws_byt
   if (status != NK_OK || splits == 1) return status;
   SplitReduce r{};
   r.partial = p.partial;
+  r.ldp = p.ldp;
   r.splits = splits;
   r.M = M;
   r.N = c.F;

@@ -145,7 +145,8 @@ size_t simt_gemm_ws(int M, int N, int splits);
 
 // Fixed-order split-K reduce with the fused epilogue (warp-shuffle tree).
 struct SplitReduce {
-  const float* partial;  // [splits][M][N] dense
+  const float* partial;  // [splits][M][ldp]
+  int ldp;               // row stride of the partials (>= N)
   int splits;
   int M, N;
   float* C;

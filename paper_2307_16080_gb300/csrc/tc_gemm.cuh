@@ -55,7 +55,9 @@ struct TcParams {
   int units;
   float* C;
   int64_t ldc;
-  float* partial;         // [splits][M][N] when splits > 1
+  float* partial;         // [splits][M][ldp] when splits > 1
+  int ldp;                // row stride of a partial tile: N rounded up to 4 floats
+  int part_vec;           // partial is 16-byte aligned
   const float* bias;
   int bias_on_m, relu;
   float beta, alpha;
@@ -691,8 +693,8 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
         const int col0 = t.tn * p.bn + c0;
         if (!row_ok || col0 >= t.N) continue;
         if (p.partial) {
-          float* dst = p.partial + ((int64_t)t.split * p.M + row) * p.N + col0;
-          if (p.c_vec && col0 + 32 <= p.N) {
+          float* dst = p.partial + ((int64_t)t.split * p.M + row) * p.ldp + col0;
+          if (p.part_vec && col0 + 32 <= p.ldp) {
 #pragma unroll
             for (int j = 0; j < 32; j += 4)
               *reinterpret_cast<float4*>(dst + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);

@@ -205,7 +205,7 @@ struct Runner {
   explicit Runner(const nk_problem* pp, const nk_schedule& s) : p(pp) {
     int64_t M, N, K;
     gemm_view(p, M, N, K);
-    const size_t split_bytes = s.split_k > 1 ? (size_t)s.split_k * M * N * 4 : 0;
+    const size_t split_bytes = s.split_k > 1 ? (size_t)s.split_k * M * ((N + 3) / 4 * 4) * 4 : 0;
     if (p->op == NK_OP_MATMUL) {
       const int kind = kind_of(p->precision);
       const int esz = kind == TC_FP8 ? 1 : 2;
@@ -258,7 +258,7 @@ struct Runner {
   nk_status run(const nk_schedule& s, cudaStream_t st) {
     int64_t M, N, K;
     gemm_view(p, M, N, K);
-    const size_t wsb = s.split_k > 1 ? (size_t)s.split_k * M * N * 4 : 0;
+    const size_t wsb = s.split_k > 1 ? (size_t)s.split_k * M * ((N + 3) / 4 * 4) * 4 : 0;
     if (p->op == NK_OP_MATMUL) return tc_gemm(g, s, ws(M, N), wsb, st);
     return tc_conv(c, s, ws(M, N), wsb, st);
   }
