@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import torch
 
@@ -144,8 +145,15 @@ def _check(status: int):
         raise NkError(status, last_error())
 
 
+# The raw handle of the current stream without a torch.cuda.Stream object per
+# call, where this torch has it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -165,6 +173,48 @@ def as_nk_tensor(t: torch.Tensor) -> nk_tensor:
         d.shape[i] = t.shape[i]
         d.stride[i] = t.stride(i)
     return d
+
+
+# Marshalling of the calls made in loops.  Filling ctypes structures field by
+# field took most of a small call's time (256^3 FP32: about 20 us a call, 5 of
+# them the kernel); the same bytes packed in one go pass as void pointers to a
+# second set of function objects, beside the typed ones of SIGNATURES.
+_TENSOR = struct.Struct("@Pii8q")        # nk_tensor
+_EPILOGUE = struct.Struct("@Piiff3P")    # nk_epilogue
+_PAIR, _QUAD = struct.Struct("@2q"), struct.Struct("@4q")
+assert _TENSOR.size == ctypes.sizeof(nk_tensor)
+_packed_fns = {}
+
+
+def _packed(name):
+    """The entry point `name` with every pointer argument a void pointer."""
+    f = _packed_fns.get(name)
+    if f is None:
+        res, args = SIGNATURES[name]
+        f = lib()[name]
+        f.restype = res
+        f.argtypes = [_P if isinstance(a, type) and issubclass(a, ctypes._Pointer) else a for a in args]
+        _packed_fns[name] = f
+    return f
+
+
+def _tensor_bytes(t: torch.Tensor) -> bytes:
+    """t as the bytes of an nk_tensor (as_nk_tensor's values)."""
+    n, shape, stride = t.dim(), t.shape, t.stride()
+    if n > 4:
+        raise ValueError("rank > 4")
+    pad = (0,) * (4 - n)
+    return _TENSOR.pack(t.data_ptr() if t.numel() else 0, _DT[t.dtype], n, *shape, *pad, *stride, *pad)
+
+
+def _epilogue_arg(bias, relu, accumulate, scale_a, scale_b, ew, pro_a, pro_b):
+    """(argument, owner): an nk_epilogue for one call, alive as long as owner."""
+    if ew is None and pro_a is None and pro_b is None:
+        e = _EPILOGUE.pack(bias.data_ptr() if bias is not None else 0, int(bool(relu)), int(bool(accumulate)),
+                           float(scale_a), float(scale_b), 0, 0, 0)
+        return e, e
+    e = _epi(bias, relu, accumulate, scale_a, scale_b, ew, pro_a, pro_b)
+    return ctypes.addressof(e), e
 
 
 def _sched(schedule):
@@ -218,9 +268,8 @@ def _epi(bias, relu, accumulate, scale_a, scale_b, ew=None, pro_a=None, pro_b=No
 
 def nk_matmul_workspace_size(A, B, C, precision="f32", schedule=None) -> int:
     n = ctypes.c_size_t(0)
-    ta, tb, tc = as_nk_tensor(A), as_nk_tensor(B), as_nk_tensor(C)
-    _check(lib().nk_matmul_workspace_size(ctypes.byref(ta), ctypes.byref(tb), ctypes.byref(tc),
-                                          PREC[precision], _sched(schedule), ctypes.byref(n)))
+    _check(_packed("nk_matmul_workspace_size")(_tensor_bytes(A), _tensor_bytes(B), _tensor_bytes(C), PREC[precision],
+                                               _sched(schedule), ctypes.byref(n)))
     return n.value
 
 
@@ -234,13 +283,16 @@ def nk_matmul(A, B, C, precision="f32", bias=None, relu=False, accumulate=False,
               scale_b=1.0, schedule=None, ws=None, stream=None, ew=None, pro_a=None, pro_b=None):
     """C = ew(ReLU?(accumulate*C + alpha*(pro_a(A) @ pro_b(B)) + bias)) through
     nk_matmul; ew / pro_a / pro_b are program step lists (make_ew_program)."""
-    ta, tb, tc = as_nk_tensor(A), as_nk_tensor(B), as_nk_tensor(C)
+    ta, tb, tc = _tensor_bytes(A), _tensor_bytes(B), _tensor_bytes(C)
+    sched, prec = _sched(schedule), PREC[precision]
     if ws is None:
-        ws = workspace(nk_matmul_workspace_size(A, B, C, precision, schedule), C.device)
-    e = _epi(bias, relu, accumulate, scale_a, scale_b, ew, pro_a, pro_b)
-    _check(lib().nk_matmul(ctypes.byref(ta), ctypes.byref(tb), ctypes.byref(tc), PREC[precision],
-                           ctypes.byref(e), _sched(schedule), ws.data_ptr() if ws is not None else None,
-                           ws.numel() if ws is not None else 0, _stream(stream)))
+        n = ctypes.c_size_t(0)
+        _check(_packed("nk_matmul_workspace_size")(ta, tb, tc, prec, sched, ctypes.byref(n)))
+        ws = workspace(n.value, C.device)
+    e, owner = _epilogue_arg(bias, relu, accumulate, scale_a, scale_b, ew, pro_a, pro_b)
+    _check(_packed("nk_matmul")(ta, tb, tc, prec, e, sched, ws.data_ptr() if ws is not None else None,
+                                ws.numel() if ws is not None else 0, _stream(stream)))
+    del owner
     return C
 
 
@@ -251,13 +303,16 @@ def _conv_args(stride, dilation, pad):
     return st, dl, pd
 
 
+def _conv_bytes(stride, dilation, pad):
+    return _PAIR.pack(*stride), _PAIR.pack(*dilation), _QUAD.pack(*pad)
+
+
 def nk_conv2d_workspace_size(I, W, O, stride=(1, 1), dilation=(1, 1), pad=(0, 0, 0, 0),
                              precision="f32", schedule=None) -> int:
     n = ctypes.c_size_t(0)
-    ti, tw, to = as_nk_tensor(I), as_nk_tensor(W), as_nk_tensor(O)
-    st, dl, pd = _conv_args(stride, dilation, pad)
-    _check(lib().nk_conv2d_workspace_size(ctypes.byref(ti), ctypes.byref(tw), ctypes.byref(to), st, dl, pd,
-                                          PREC[precision], _sched(schedule), ctypes.byref(n)))
+    _check(_packed("nk_conv2d_workspace_size")(_tensor_bytes(I), _tensor_bytes(W), _tensor_bytes(O),
+                                               *_conv_bytes(stride, dilation, pad), PREC[precision], _sched(schedule),
+                                               ctypes.byref(n)))
     return n.value
 
 
@@ -268,15 +323,18 @@ def nk_conv2d_nhwc_hwcf(I, W, O, stride=(1, 1), dilation=(1, 1), pad=(0, 0, 0, 0
     programs are step lists (make_ew_program), the zero padding stays 0.
     scale_i, scale_w: the quantisation scales of E4M3 operands the caller
     quantised (read only for those)."""
-    ti, tw, to = as_nk_tensor(I), as_nk_tensor(W), as_nk_tensor(O)
-    st, dl, pd = _conv_args(stride, dilation, pad)
+    ti, tw, to = _tensor_bytes(I), _tensor_bytes(W), _tensor_bytes(O)
+    st, dl, pd = _conv_bytes(stride, dilation, pad)
+    sched, prec = _sched(schedule), PREC[precision]
     if ws is None:
-        ws = workspace(nk_conv2d_workspace_size(I, W, O, stride, dilation, pad, precision, schedule), O.device)
-    e = _epi(bias, relu, accumulate, scale_i, scale_w, ew, pro_i, pro_w)
-    _check(lib().nk_conv2d_nhwc_hwcf(ctypes.byref(ti), ctypes.byref(tw), ctypes.byref(to), st, dl, pd,
-                                     PREC[precision], ctypes.byref(e), _sched(schedule),
-                                     ws.data_ptr() if ws is not None else None,
-                                     ws.numel() if ws is not None else 0, _stream(stream)))
+        n = ctypes.c_size_t(0)
+        _check(_packed("nk_conv2d_workspace_size")(ti, tw, to, st, dl, pd, prec, sched, ctypes.byref(n)))
+        ws = workspace(n.value, O.device)
+    e, owner = _epilogue_arg(bias, relu, accumulate, scale_i, scale_w, ew, pro_i, pro_w)
+    _check(_packed("nk_conv2d_nhwc_hwcf")(ti, tw, to, st, dl, pd, prec, e, sched,
+                                          ws.data_ptr() if ws is not None else None,
+                                          ws.numel() if ws is not None else 0, _stream(stream)))
+    del owner
     return O
 
 
@@ -324,11 +382,10 @@ def quantize_nhwc_fp8(I, stream=None):
 def nk_conv2d_nchw_fchw(I, K, O, stride=(1, 1), dilation=(1, 1), pad=(0, 0, 0, 0), bias=None, relu=False,
                         accumulate=False, stream=None, ew=None):
     """Direct NCHW / FCHW convolution (Listing "2dnchwconv" layout)."""
-    ti, tk, to = as_nk_tensor(I), as_nk_tensor(K), as_nk_tensor(O)
-    st, dl, pd = _conv_args(stride, dilation, pad)
-    e = _epi(bias, relu, accumulate, 1.0, 1.0, ew)
-    _check(lib().nk_conv2d_nchw_fchw(ctypes.byref(ti), ctypes.byref(tk), ctypes.byref(to), st, dl, pd,
-                                     ctypes.byref(e), _stream(stream)))
+    e, owner = _epilogue_arg(bias, relu, accumulate, 1.0, 1.0, ew, None, None)
+    _check(_packed("nk_conv2d_nchw_fchw")(_tensor_bytes(I), _tensor_bytes(K), _tensor_bytes(O),
+                                          *_conv_bytes(stride, dilation, pad), e, _stream(stream)))
+    del owner
     return O
 
 
