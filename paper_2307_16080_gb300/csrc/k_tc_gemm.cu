@@ -579,6 +579,27 @@ nk_schedule grouped_schedule(const nk_schedule* user) {
   return s;
 }
 
+// The built-in tile of a grouped GEMM: 128 x 128 with the deepest ring, or 128
+// x 256 with four stages where the groups fill it.  In units of a 64-deep K
+// block of a 128 x 256 tile, a 128 x 128 one costs 0.72 (its MMAs are not half
+// as long), and the tiles' epilogues 4 and 2.  Measured, 128 x 128 / 128 x 256,
+// us: 512 groups of 32 to 2048 222.7 / 189.9, 512 to 1024 75.5 / 69.7, 32 to
+// 2048 26.3 / 22.7; 512 groups of 32 to 512 32.1 / 33.8 (stays 128 x 128).
+nk_schedule grouped_gemm_schedule(int G, const nk_gemm_group* groups, const nk_schedule* user) {
+  if (user && (user->tile_m || user->tile_n || user->tile_k || user->cluster || user->stages || user->split_k))
+    return grouped_schedule(user);
+  double square = 0, wide = 0;
+  for (int g = 0; g < G; ++g) {
+    const nk_gemm_group& q = groups[g];
+    if (q.M < 1 || q.N < 1 || q.K < 1) continue;   // refused below
+    const double tm = (q.M + 127) / 128, kb = (q.K + 63) / 64;
+    square += tm * ((q.N + 127) / 128) * (0.72 * kb + 2);
+    wide += tm * ((q.N + 255) / 256) * (kb + 4);
+  }
+  if (wide < square) return nk_schedule{128, 256, 64, 1, 4, 1};
+  return grouped_schedule(nullptr);
+}
+
 // Fills `host` (grouped_bytes(G) bytes) with the table for a device buffer at
 // `dev_base`, and the launch parameters.
 nk_status build_grouped(int G, const nk_gemm_group* groups, int precision, const nk_schedule* user,
@@ -587,7 +608,7 @@ nk_status build_grouped(int G, const nk_gemm_group* groups, int precision, const
   if (G > 0 && !groups) return fail(NK_ERR_INVALID_ARG, "groups is NULL");
   if (precision != NK_PREC_BF16)
     return fail(NK_ERR_UNSUPPORTED, "grouped GEMM runs BF16 operands (NK_PREC_BF16) only");
-  const nk_schedule s = grouped_schedule(user);
+  const nk_schedule s = grouped_gemm_schedule(G, groups, user);
   // tile_m 128 on one CTA, or tile_m 256 on a CTA pair (each CTA holds its
   // 128 rows of A and half of the B tile)
   const bool pair = s.tile_m == 256 && s.cluster == 2;
