@@ -264,6 +264,21 @@ static __device__ __forceinline__ void ew_apply(const EwProg& e, float* buf, int
   for (int i = 0; i < e.n; ++i) ew_op_buf(e.op[i], e.a[i], e.b[i], e.t[i] + off0, buf, n);
 }
 
+// v[j] += bias[j] for 32 columns that all exist: eight 16-byte loads (the same
+// for every lane) where the bias allows them, 32 scalar ones else.
+__device__ __forceinline__ void add_bias32(const float* bias, float (&v)[32]) {
+  if ((reinterpret_cast<uintptr_t>(bias) & 15) == 0) {
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) {
+      const float4 b = __ldg(reinterpret_cast<const float4*>(bias + j));
+      v[j] += b.x; v[j + 1] += b.y; v[j + 2] += b.z; v[j + 3] += b.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] += __ldg(bias + j);
+  }
+}
+
 // 32-byte stores (one whole L2 sector per thread; the address must be
 // 32-byte aligned).  The epilogues write one output row per lane, so a warp
 // store touches 32 rows: with 16-byte stores each row's sector arrives in

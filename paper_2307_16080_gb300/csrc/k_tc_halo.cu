@@ -411,12 +411,10 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
             // Full 32-column segment, no accumulate, and no program or the
             // residual program ADD t, RELU (inline, same FP32 steps as the
             // interpreter): one code path for FP32 and BF16 outputs.
+            if (p.bias) add_bias32(p.bias + col0, v);
+            if (p.relu) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              float xv = v[j];
-              if (p.bias) xv += __ldg(p.bias + col0 + j);
-              if (p.relu) xv = (xv > 0.f || xv != xv) ? xv : 0.f;
-              v[j] = xv;
+              for (int j = 0; j < 32; ++j) v[j] = (v[j] > 0.f || v[j] != v[j]) ? v[j] : 0.f;
             }
             if constexpr (RES) {
               const float4* tr = reinterpret_cast<const float4*>(p.ew.t[0] + orow_off + col0);
@@ -847,7 +845,14 @@ nk_schedule tc_halo_default_schedule(const ConvGeom& g, int F, int sms, bool* ok
     // 32x56x56x64 (896 tiles); at 8x56x56x64 (224 tiles) one buffer stays
     // ahead, 8.0 against 8.3 us.
     const nk_schedule d{256, 64, cb * g.kh, 1, 2, 1};
-    if (units >= 4 * (int64_t)sms && halo_schedule_valid(g, F, d, kind)) s = d;
+    if (units >= 4 * (int64_t)sms && halo_schedule_valid(g, F, d, kind)) {
+      // With more than one channel block and more than one filter tile that
+      // many units are faster on CTA pairs, per tap (tc_conv_default_schedule):
+      // 128x28x28x128 50.3 / 33.3 us, 128x14x14x256 55.3 / 39.3, 32x40x40x160
+      // 59.4 / 44.4, 128x33x33x72 193 / 79.
+      if (kind == TC_BF16 && g.c > 64 && F > 64) return best;
+      s = d;
+    }
     *ok = true;
     return s;
   }

@@ -712,11 +712,11 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
             // steps): one code path for FP32 and BF16 outputs.
             const int64_t off = (int64_t)row * t.ldc + col0;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              float x = alpha * v[j];
-              if (t.bias) x += __ldg(t.bias + col0 + j);
-              if (t.relu) x = (x > 0.f || x != x) ? x : 0.f;
-              v[j] = x;
+            for (int j = 0; j < 32; ++j) v[j] *= alpha;
+            if (t.bias) add_bias32(t.bias + col0, v);
+            if (t.relu) {
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] = (v[j] > 0.f || v[j] != v[j]) ? v[j] : 0.f;
             }
             if (p.resid) {
               const float4* tr = reinterpret_cast<const float4*>(p.ew.t[0] + off);
