@@ -275,13 +275,12 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
         b[2 * h].v = q.x;
         b[2 * h + 1].v = q.y;
       }
-      f2 aa[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) aa[i] = f2_set(a[i]);
+      for (int i = 0; i < 8; ++i) {
+        const f2 aa = f2_set(a[i]);
 #pragma unroll
-      for (int j = 0; j < TN / 2; ++j)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i][j] = f2_fma(aa[i], b[j], acc[i][j]);
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = f2_fma(aa, b[j], acc[i][j]);
+      }
     };
     if constexpr (AMK) {
 #pragma unroll
@@ -690,8 +689,8 @@ inline bool al16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) =
 // its units (tiles x slices) at the rate the tile's shape reaches, each unit
 // costs about a microsecond to fill and drain, and a cluster's exchange 1.6;
 // clusters of eight 128-row tiles pack badly.  The constants are fitted to
-// every combination timed on 23 shapes (products from 64^3 to 4096^3 and eight
-// convolutions), where the choice is 1.3 % off the best on average and 11 % at
+// every combination timed on 27 shapes (products from 64^3 to 4096^3 and eight
+// convolutions), where the choice is 1.9 % off the best on average and 12 % at
 // worst.  Examples, us (tile / cluster): 256^3 64x64 / 1 12.3, / 8 5.3; 1024^3
 // 128x128 / 1 103, / 4 53; 1531 x 2047 x 1021 128x128 / 1 194, / 4 150;
 // 8x56x56x64 3x3 64x64 / 1 71, 128x64 / 2 52.
@@ -703,7 +702,7 @@ Choice choose(int M, int N, int K, int sms, bool may_split) {
     int bm, bn, resident;
     double gflop_us;   // per SM
   };
-  static const Tile kTiles[] = {{128, 128, 2, 0.366}, {128, 64, 3, 0.359}, {64, 64, 2, 0.355}};
+  static const Tile kTiles[] = {{128, 128, 2, 0.366}, {128, 64, 3, 0.352}, {64, 64, 2, 0.369}};
   Choice best{128, 128, 1};
   double best_t = 1e30;
   for (const Tile& t : kTiles) {
@@ -714,11 +713,11 @@ Choice choose(int M, int N, int K, int sms, bool may_split) {
       // units of the busiest SM: whole ones while all are resident at once,
       // then the average and about half a set in the last wave
       const double u = units <= (int64_t)sms * t.resident ? (double)((units + sms - 1) / sms)
-                                                          : (double)units / sms + 0.59 * t.resident;
+                                                          : (double)units / sms + 0.51 * t.resident;
       const double warps = u * (t.bn == 128 ? 8 : 4);
-      const double fill = warps < 8 ? 0.575 : warps < 12 ? 0.864 : 1.0;   // too few to keep the FMA pipes busy
+      const double fill = warps < 8 ? 0.624 : warps < 12 ? 0.864 : 1.0;   // too few to keep the FMA pipes busy
       const double kc = ((K + cs - 1) / cs + BK - 1) / BK * BK;
-      const double pack = t.bm == 128 ? (cs == 8 ? 1.276 : cs == 4 ? 0.915 : 1.0) : 1.0;
+      const double pack = t.bm == 128 ? (cs == 8 ? 1.276 : cs == 4 ? 0.882 : 1.0) : 1.0;
       const double us = u * (2e-6 * t.bm * t.bn * kc * pack / (t.gflop_us * fill) + 1.064) + (cs > 1 ? 1.642 : 0.0);
       if (us < best_t) {
         best_t = us;
@@ -760,7 +759,9 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
   const ConvGeom& cg = p.conv;
   const bool far = p.is_conv && (cg.h + cg.pt + cg.kh * cg.dh > 32000 || cg.w + cg.pl + cg.kw * cg.dw > 32000 ||
                                  cg.oh * (int64_t)cg.sh > 32000 || cg.ow * (int64_t)cg.sw > 32000 ||
-                                 cg.n * cg.sin_n + cg.h * cg.sin_h + cg.w * cg.sin_w >= INT32_MAX / 2);
+                                 cg.n * cg.sin_n + (cg.h + cg.pt + cg.kh * cg.dh) * cg.sin_h +
+                                         (cg.w + cg.pl + cg.kw * cg.dw) * cg.sin_w >=
+                                     INT32_MAX / 2);
   if (p.pro_a.n || p.pro_b.n || p.ew.n || far) {
     if (tile == 0) tile = (int64_t)((p.M + 127) / 128) * ((p.N + 127) / 128) < 152 ? 64 : 128;
     const dim3 grid((p.N + tile - 1) / tile, (p.M + tile - 1) / tile, splits);
