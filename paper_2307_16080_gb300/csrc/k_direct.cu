@@ -8,20 +8,21 @@
 // HBM: each input element is read once through a shared-memory halo tile,
 // each output element written once with 128-bit stores.
 //
-// Two kernels:
+// Three kernels:
 //   direct_rows_kernel (stride 1, dilation 1, 1x1 / 3x3 / 5x5 filters): each
 //     thread owns 4 consecutive output columns of ROWS consecutive rows for
-//     up to CO_G output channels and walks down the ROWS + KH - 1 input rows
+//     up to four output channels and walks down the ROWS + KH - 1 input rows
 //     it needs, one register segment of 4 + KW - 1 values per row (each input
 //     row feeds every output row and tap that uses it), so the input is read
-//     from DRAM once, with no shared memory and no index division; the
-//     filter taps of an input channel sit in registers.  Outputs leave as
-//     16-byte (or, on rows that are only 8-byte aligned, 8-byte) stores.
-//   direct_stream_kernel (the same filters, one input channel -- the tuning
-//     experiment's Ci = 1): as above, but a thread walks `rpt` output rows
-//     keeping only KH rotating accumulator rows; an output row is stored as
-//     soon as its last tap row has arrived, so the halo rows are amortised
-//     over many rows and the stores spread through the loop.
+//     from DRAM once, with no shared memory; the filter taps of an input
+//     channel sit in registers.  Outputs leave as 16-byte stores (8-byte or
+//     single ones on rows that are not aligned to them).
+//   direct_stream_kernel (1x1 to one output channel and 3x3 filters, one input
+//     channel -- the tuning experiment's Ci = 1 -- on large images): as above,
+//     but a thread walks `rpt` output rows keeping only KH rotating accumulator
+//     rows; an output row is stored as soon as its last tap row has arrived, so
+//     the halo rows are amortised over many rows and the stores spread through
+//     the loop.
 //   direct_conv_kernel (any stride / dilation / filter up to 64 taps): a CTA
 //     computes a 16 x 64 output tile of one image for up to 8 output
 //     channels from a halo tile staged in shared memory, one input channel
@@ -143,82 +144,120 @@ __global__ void __launch_bounds__(THREADS) direct_conv_kernel(const __grid_const
   }
 }
 
-// Input segment x[0..SEG) = row ih, columns iw0 .. iw0+SEG-1, zero outside.
+// Input segment x[0..SEG) of a row that starts at src; wi is the column of
+// src[0], columns outside [0, W) are zero.  vec: the whole warp's segments are
+// 16-byte aligned and inside the row.
 template <int SEG>
-__device__ __forceinline__ void load_segment(const float* src, int64_t sIh, int H, int W, int ih, int iw0,
-                                             float (&x)[SEG]) {
-  if (ih < 0 || ih >= H) {
-#pragma unroll
-    for (int j = 0; j < SEG; ++j) x[j] = 0.f;
-    return;
-  }
-  const float* row = src + (int64_t)ih * sIh;
-  if (iw0 >= 0 && iw0 + SEG <= W) {
-    const float* q = row + iw0;
-    if (SEG >= 4 && (reinterpret_cast<uintptr_t>(q) & 15) == 0) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(q));
-      x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-      if constexpr (SEG == 6) {
-        const float2 b = __ldg(reinterpret_cast<const float2*>(q + 4));
-        x[4] = b.x; x[5] = b.y;
-      } else if constexpr (SEG == 8) {
-        const float4 b = __ldg(reinterpret_cast<const float4*>(q + 4));
-        x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-      } else {
-#pragma unroll
-        for (int j = 4; j < SEG; ++j) x[j] = __ldg(q + j);
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < SEG; ++j) x[j] = __ldg(q + j);
+__device__ __forceinline__ void load_row(const float* src, bool vec, int wi, int W, float (&x)[SEG]) {
+  if (SEG >= 4 && vec) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(src));
+    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+    if constexpr (SEG == 6) {
+      const float2 t = __ldg(reinterpret_cast<const float2*>(src + 4));
+      x[4] = t.x; x[5] = t.y;
+    } else if constexpr (SEG == 8) {
+      const float4 t = __ldg(reinterpret_cast<const float4*>(src + 4));
+      x[4] = t.x; x[5] = t.y; x[6] = t.z; x[7] = t.w;
     }
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int j = 0; j < SEG; ++j) {
-    const int iw = iw0 + j;
-    x[j] = (iw >= 0 && iw < W) ? __ldg(row + iw) : 0.f;
+    for (int j = 0; j < SEG; ++j) x[j] = (unsigned)(wi + j) < (unsigned)W ? __ldg(src + j) : 0.f;
   }
 }
 
-template <int KH, int KW, int CO_G, int ROWS>
-__global__ void __launch_bounds__(128) direct_rows_kernel(const __grid_constant__ Direct p) {
+// Epilogue and store of a lane's four outputs at d, on a row that starts s
+// floats before a 16-byte boundary; full: every lane of the warp has all four.
+template <bool PLAIN>
+__device__ __forceinline__ void finish_row(const Direct& p, float* d, int s, bool full, int wo, float bias,
+                                           const float (&acc)[4]) {
+  float v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float o = acc[j];
+    if constexpr (!PLAIN)
+      if (p.beta != 0.f && wo + j < p.OW) o = fmaf(p.beta, d[j], o);
+    o += bias;
+    if constexpr (!PLAIN)
+      if (p.relu) o = (o > 0.f || o != o) ? o : 0.f;
+    v[j] = o;
+  }
+  if (full && s == 0) {
+    *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
+  } else if (full && s == 2) {
+    *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
+    *reinterpret_cast<float2*>(d + 2) = make_float2(v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (full || wo + j < p.OW) d[j] = v[j];
+  }
+}
+
+// CTAs per SM that direct_rows_kernel's registers have to leave room for: its
+// loads are hidden by other warps alone.  16 x 3 x 1280 x 1280 -> 3, 3 x 3: 219 us
+// at seven CTAs, 286 with the registers the compiler would take; 16 x 3 x 700 x
+// 800 -> 4, 5 x 5 in pairs of channels: 162 at eight, 176 at six; 8 x 3 x 640 x 640
+// -> 3, 5 x 5: 57 at four, 72 at five (spills).
+constexpr int rows_ctas(int kh, int co) {
+  return kh == 5 ? (co == 1 ? 10 : co == 2 ? 8 : 4)
+       : kh == 3 ? (co == 1 ? 12 : co == 2 ? 9 : co == 3 ? 7 : 5)
+                 : (co <= 2 ? 16 : co == 3 ? 12 : 9);
+}
+
+// Blocks of rows: a thread owns four columns of ROWS output rows and walks the
+// ROWS + KH - 1 input rows of one channel after another.  Issue slots bound it
+// like the kernel below, so it has the same exact CO, PLAIN, and alignment
+// settled once.
+template <int KH, int KW, int CO, int ROWS, bool PLAIN>
+__global__ void __launch_bounds__(128, rows_ctas(KH, CO)) direct_rows_kernel(const __grid_constant__ Direct p, int cols) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
   constexpr int SEG = 4 + KW - 1;
   constexpr int TAPS = KH * KW;
-  const int wo = blockIdx.x * 512 + threadIdx.x * 4;   // first of this thread's 4 output columns
-  const int ho0 = blockIdx.y * ROWS;
-  const int groups = (p.CO + CO_G - 1) / CO_G;
-  const int n = blockIdx.z / groups;
-  const int co0 = (blockIdx.z % groups) * CO_G;
-  const int ncog = min(CO_G, p.CO - co0);
-  if (wo >= p.OW) return;
-  float acc[ROWS][CO_G][4];
+  const int lane = threadIdx.x & 31;
+  const int by = blockIdx.x / cols;   // grid.x: `cols` blocks of columns for each block of rows
+  const int wo = (blockIdx.x - by * cols) * 512 + threadIdx.x * 4;   // first of this thread's 4 output columns
+  const int ho0 = by * ROWS;
+  const int groups = (p.CO + CO - 1) / CO;
+  const int n = blockIdx.y / groups;
+  const int co0 = (blockIdx.y % groups) * CO;
+  const int ncog = min(CO, p.CO - co0);
+  if (wo - lane * 4 >= p.OW) return;   // whole warps: the stores shuffle
+  float acc[ROWS][CO][4];
 #pragma unroll
   for (int r = 0; r < ROWS; ++r)
 #pragma unroll
-    for (int c = 0; c < CO_G; ++c)
+    for (int c = 0; c < CO; ++c)
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[r][c][j] = 0.f;
-  for (int ci = 0; ci < p.CI; ++ci) {
-    float w[CO_G][TAPS];
+  const float* src = p.I + n * p.sIn + (int64_t)(ho0 - p.pt) * p.sIh + (wo - p.pl);
+  const bool vec = __all_sync(0xffffffffu, wo - p.pl >= 0 && wo - p.pl + SEG <= p.W && (p.sIh & 3) == 0 &&
+                                               ((p.sIc & 3) == 0 || p.CI == 1) &&
+                                               (reinterpret_cast<uintptr_t>(src) & 15) == 0);
+#pragma unroll 1
+  for (int ci = 0; ci < p.CI; ++ci, src += p.sIc) {
+    float w[CO][TAPS];
 #pragma unroll
-    for (int c = 0; c < CO_G; ++c)
+    for (int c = 0; c < CO; ++c)
 #pragma unroll
       for (int t = 0; t < TAPS; ++t)
         w[c][t] = c < ncog ? __ldg(p.Kr + ((int64_t)(co0 + c) * p.CI + ci) * TAPS + t) : 0.f;
-    const float* src = p.I + n * p.sIn + ci * p.sIc;
 #pragma unroll
     for (int r = 0; r < ROWS + KH - 1; ++r) {   // input row ho0 + r - pt
       float x[SEG];
-      load_segment<SEG>(src, p.sIh, p.H, p.W, ho0 + r - p.pt, wo - p.pl, x);
+      const int ih = ho0 + r - p.pt;
+      if ((unsigned)ih < (unsigned)p.H) {
+        load_row<SEG>(src + (int64_t)r * p.sIh, vec, wo - p.pl, p.W, x);
+      } else {
+#pragma unroll
+        for (int j = 0; j < SEG; ++j) x[j] = 0.f;
+      }
 #pragma unroll
       for (int kh = 0; kh < KH; ++kh) {
         const int orow = r - kh;   // the output row this input row meets through tap row kh
         if (orow < 0 || orow >= ROWS) continue;
 #pragma unroll
-        for (int c = 0; c < CO_G; ++c)
+        for (int c = 0; c < CO; ++c)
 #pragma unroll
           for (int kw = 0; kw < KW; ++kw)
 #pragma unroll
@@ -226,64 +265,19 @@ __global__ void __launch_bounds__(128) direct_rows_kernel(const __grid_constant_
       }
     }
   }
+  const bool full = __all_sync(0xffffffffu, wo + 3 < p.OW);
+  float* dst = p.O + n * p.sOn + (int64_t)co0 * p.sOc + (int64_t)ho0 * p.sOh + wo;
+  // floats into a 16-byte word at which a row starts: wo is a multiple of 4
+  const int at = (int)((reinterpret_cast<uintptr_t>(p.O) >> 2) + n * p.sOn + co0 * p.sOc + ho0 * p.sOh);
 #pragma unroll
   for (int r = 0; r < ROWS; ++r) {
-    const int ho = ho0 + r;
-    if (ho >= p.OH) break;
+    if (ho0 + r >= p.OH) break;
 #pragma unroll
-    for (int c = 0; c < CO_G; ++c) {
+    for (int c = 0; c < CO; ++c) {
       if (c >= ncog) break;
-      float* dst = p.O + n * p.sOn + (int64_t)(co0 + c) * p.sOc + (int64_t)ho * p.sOh + wo;
-      const float b = p.bias ? __ldg(p.bias + co0 + c) : 0.f;
-      float v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float o = acc[r][c][j];
-        if (p.beta != 0.f && wo + j < p.OW) o = fmaf(p.beta, dst[j], o);
-        o += b;
-        if (p.relu) o = (o > 0.f || o != o) ? o : 0.f;
-        v[j] = o;
-      }
-      const uintptr_t a = reinterpret_cast<uintptr_t>(dst);
-      if (wo + 3 < p.OW && (a & 15) == 0) {
-        *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-      } else if (wo + 3 < p.OW && (a & 7) == 0) {
-        *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
-        *reinterpret_cast<float2*>(dst + 2) = make_float2(v[2], v[3]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (wo + j < p.OW) dst[j] = v[j];
-      }
+      const int s = -(at + c * (int)(p.sOc & 3) + r * (int)(p.sOh & 3)) & 3;
+      finish_row<PLAIN>(p, dst + c * p.sOc + r * p.sOh, s, full, wo, p.bias ? __ldg(p.bias + co0 + c) : 0.f, acc[r][c]);
     }
-  }
-}
-
-// Stores a warp's 128 consecutive outputs of one row and channel, four a lane,
-// to a row that starts s floats before a 16-byte boundary (the same s for the
-// whole warp) or ends inside the warp.  A lane stores its last 4 - s values
-// and its neighbour's first s as one aligned 16-byte word, so the warp writes
-// whole sectors; the ends of the row, and lane 0's first s values, go out one
-// by one.  Out of line: the unrolled loop keeps the two common cases.
-__device__ __noinline__ void store_shifted(float* dst, int s, int wo, int OW, float v0, float v1, float v2, float v3) {
-  const int lane = threadIdx.x & 31;
-  const float n0 = __shfl_down_sync(0xffffffffu, v0, 1);
-  const float n1 = __shfl_down_sync(0xffffffffu, v1, 1);
-  const float n2 = __shfl_down_sync(0xffffffffu, v2, 1);
-  if ((s == 0 || lane < 31) && wo + s + 3 < OW) {
-    *reinterpret_cast<float4*>(dst + s) =
-        make_float4(s == 0 ? v0 : s == 1 ? v1 : s == 2 ? v2 : v3, s == 0 ? v1 : s == 1 ? v2 : s == 2 ? v3 : n0,
-                    s == 0 ? v2 : s == 1 ? v3 : s == 2 ? n0 : n1, s == 0 ? v3 : s == 1 ? n0 : s == 2 ? n1 : n2);
-  } else {
-    if (s <= 0 && wo < OW) dst[0] = v0;
-    if (s <= 1 && wo + 1 < OW) dst[1] = v1;
-    if (s <= 2 && wo + 2 < OW) dst[2] = v2;
-    if (wo + 3 < OW) dst[3] = v3;
-  }
-  if (s && (lane == 0 || wo + s - 1 >= OW)) {   // no lane before this one stored these
-    if (wo < OW) dst[0] = v0;
-    if (s > 1 && wo + 1 < OW) dst[1] = v1;
-    if (s > 2 && wo + 2 < OW) dst[2] = v2;
   }
 }
 
@@ -297,7 +291,9 @@ __device__ __noinline__ void store_shifted(float* dst, int s, int wo, int OW, fl
 // ReLU out, and range and alignment are settled once per thread where they can
 // be.  16 x 1280 x 1280, 3 x 3, 1 -> 3 channels (418 MB): 330 instructions per
 // warp and row, four channels computed for three and 8-byte stores on every
-// other row took 123 us; now 84 us.
+// other row took 123 us; now 69 us, 90 % of the copy rate.  Rows on odd floats: single stores; putting
+// two lanes' values together into aligned 16-byte ones costs more issue slots
+// than it saves (16 x 1000 x 1001 1 -> 4, 3 x 3: 91 us so, 68 us now).
 template <int KH, int KW, int CO, bool PLAIN>
 __global__ void __launch_bounds__(128) direct_stream_kernel(const __grid_constant__ Direct p, int rpt) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
@@ -345,20 +341,7 @@ __global__ void __launch_bounds__(128) direct_stream_kernel(const __grid_constan
   auto load = [&](int r, float (&x)[SEG]) {
     const int ih = ho0 + r - p.pt;
     if (r < nin && ih >= 0 && ih < p.H) {
-      if (SEG >= 4 && vec) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(src));
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-        if constexpr (SEG == 6) {
-          const float2 t = __ldg(reinterpret_cast<const float2*>(src + 4));
-          x[4] = t.x; x[5] = t.y;
-        } else if constexpr (SEG == 8) {
-          const float4 t = __ldg(reinterpret_cast<const float4*>(src + 4));
-          x[4] = t.x; x[5] = t.y; x[6] = t.z; x[7] = t.w;
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < SEG; ++j) x[j] = (unsigned)(wo - p.pl + j) < (unsigned)p.W ? __ldg(src + j) : 0.f;
-      }
+      load_row<SEG>(src, vec, wo - p.pl, p.W, x);
     } else {
 #pragma unroll
       for (int j = 0; j < SEG; ++j) x[j] = 0.f;
@@ -396,27 +379,7 @@ __global__ void __launch_bounds__(128) direct_stream_kernel(const __grid_constan
 #pragma unroll
       for (int c = 0; c < CO; ++c) {
         if (c >= ncog) break;
-        float* d = dst + c * p.sOc;
-        float v[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float o = acc[slot][c][j];
-          if constexpr (!PLAIN)
-            if (p.beta != 0.f && wo + j < p.OW) o = fmaf(p.beta, d[j], o);
-          o += bias[c];
-          if constexpr (!PLAIN)
-            if (p.relu) o = (o > 0.f || o != o) ? o : 0.f;
-          v[j] = o;
-        }
-        const int s = -(at + c * sOc4) & 3;
-        if (full && s == 0) {
-          *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
-        } else if (full && s == 2) {
-          *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
-          *reinterpret_cast<float2*>(d + 2) = make_float2(v[2], v[3]);
-        } else {
-          store_shifted(d, s, wo, p.OW, v[0], v[1], v[2], v[3]);
-        }
+        finish_row<PLAIN>(p, dst + c * p.sOc, -(at + c * sOc4) & 3, full, wo, bias[c], acc[slot][c]);
       }
       dst += p.sOh;
       at += sOh4;
@@ -424,52 +387,91 @@ __global__ void __launch_bounds__(128) direct_stream_kernel(const __grid_constan
   }
 }
 
-// Four output channels per thread keep the accumulators and taps in
-// registers (eight with a 5 x 5 filter would spill).
-template <int KH, int KW>
-nk_status launch_rows(const Direct& p, cudaStream_t st) {
-  constexpr int ROWS = 4, CO_R = 4;
-  const int groups = (p.CO + CO_R - 1) / CO_R;
-  if ((int64_t)p.N * groups > 65535) return fail(NK_ERR_UNSUPPORTED, "batch x channel groups too large");
-  dim3 grid((unsigned)((p.OW + 511) / 512), (unsigned)((p.OH + ROWS - 1) / ROWS), (unsigned)(p.N * groups));
-  if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "output too tall");
-  (void)nk::launch_k(direct_rows_kernel<KH, KW, CO_R, ROWS>, dim3(grid), dim3(128), 0, st, 1, p);
+// Up to four output channels per thread keep the accumulators and taps in
+// registers; four with a 5 x 5 filter leave too few warps to hide the loads, so
+// they go in pairs.  Two rows per thread instead of four while four would give
+// fewer than six CTAs per SM, and for 1 x 1 filters, which have no halo rows to
+// share; then pairs of channels for 3 x 3 too.  Measured, us, a kernel of four
+// channels and four rows with loads and stores settled one by one / this: 16 x 3
+// x 1280 x 1280 -> 3, 3 x 3: 320 / 219; 8 x 3 x 640 x 640 -> 3, 5 x 5: 83 / 57;
+// 16 x 3 x 700 x 800 -> 4, 5 x 5: 218 / 162 (206 with four channels together); 1 x
+// 3 x 1000 x 1000 -> 3, 3 x 3: 12.3 / 8.7 (14.0 with four rows); 8 x 3 x 1000 x 1000
+// -> 4, 1 x 1: 62 / 42 (63 with four rows).  Six or eight rows: 268 to 275 us on the
+// first.
+template <int KH, int KW, int CO, int ROWS>
+nk_status launch_rows_co(const Direct& p, cudaStream_t st) {
+  const int cols = (p.OW + 511) / 512;
+  dim3 grid((unsigned)cols * (unsigned)((p.OH + ROWS - 1) / ROWS), (unsigned)(p.N * ((p.CO + CO - 1) / CO)));
+  if (p.beta == 0.f && !p.relu) (void)nk::launch_k(direct_rows_kernel<KH, KW, CO, ROWS, true>, grid, dim3(128), 0, st, 1, p, cols);
+  else (void)nk::launch_k(direct_rows_kernel<KH, KW, CO, ROWS, false>, grid, dim3(128), 0, st, 1, p, cols);
   return check_launch("direct_rows_kernel");
 }
 
-// One input channel: output rows per thread.  Runs short enough that the grid
-// walks the images nearly in order, long enough to amortise the KH - 1 halo
-// rows, and at least six CTAs per SM.  Measured, us for 4 / 8 / 16 / 32 / 64
-// rows: 16 x 1280 x 1280 1 -> 3, 3 x 3: 90 / 84 / 89 / 110 / 156; 5 x 5: 268 /
-// 211 / 180 / 179 / 206; 1 x 1280 x 1280, 3 x 3: 11 / 14 / 18 / 33 / 63; 16 x
-// 1000 x 1000 1 -> 4, 1 x 1: 50 / 55 / 64 / 82 / 100.
-template <int KH, int KW, int CO>
-nk_status launch_stream_co(const Direct& p, cudaStream_t st) {
-  int sms = 152;
-  nk_status s = require_device(&sms);
-  if (s != NK_OK) return s;
-  const int groups = (p.CO + CO - 1) / CO;
-  if ((int64_t)p.N * groups > 65535) return fail(NK_ERR_UNSUPPORTED, "batch x channel groups too large");
-  const int64_t ctas_per_row = (int64_t)((p.OW + 511) / 512) * p.N * groups;
-  constexpr int64_t kRows = KH == 1 ? 4 : KH == 3 ? 8 : 24;
-  int64_t rpt = (int64_t)p.OH * ctas_per_row / ((int64_t)sms * 6);
-  rpt = rpt < 4 ? 4 : rpt > kRows ? kRows : rpt;
-  if ((p.OH + rpt - 1) / rpt > 65535) rpt = 64;   // grid.y
-  dim3 grid((unsigned)((p.OW + 511) / 512), (unsigned)((p.OH + rpt - 1) / rpt), (unsigned)(p.N * groups));
-  if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "output too tall");
-  if (p.beta == 0.f && !p.relu) (void)nk::launch_k(direct_stream_kernel<KH, KW, CO, true>, grid, dim3(128), 0, st, 1, p, (int)rpt);
-  else (void)nk::launch_k(direct_stream_kernel<KH, KW, CO, false>, grid, dim3(128), 0, st, 1, p, (int)rpt);
-  return check_launch("direct_stream_kernel");
+template <int KH, int KW, int ROWS>
+nk_status launch_rows_r(const Direct& p, int co, cudaStream_t st) {
+  switch (co) {
+    case 1: return launch_rows_co<KH, KW, 1, ROWS>(p, st);
+    case 2: return launch_rows_co<KH, KW, 2, ROWS>(p, st);
+    case 3: return launch_rows_co<KH, KW, 3, ROWS>(p, st);
+    default: return launch_rows_co<KH, KW, 4, ROWS>(p, st);
+  }
 }
 
 template <int KH, int KW>
-nk_status launch_stream(const Direct& p, cudaStream_t st) {
-  switch (p.CO) {
-    case 1: return launch_stream_co<KH, KW, 1>(p, st);
-    case 2: return launch_stream_co<KH, KW, 2>(p, st);
-    case 3: return launch_stream_co<KH, KW, 3>(p, st);
-    default: return launch_stream_co<KH, KW, 4>(p, st);
+nk_status launch_rows(const Direct& p, int sms, cudaStream_t st) {
+  int co = p.CO < 4 ? p.CO : 4;
+  const int64_t blocks = (int64_t)((p.OW + 511) / 512) * ((p.OH + 3) / 4) * p.N;
+  const bool few = blocks * ((p.CO + 3) / 4) < (int64_t)sms * 6;
+  if (co == 4 && (KH == 5 || (KH == 3 && few)) && (int64_t)p.N * ((p.CO + 1) / 2) <= 65535) co = 2;
+  if constexpr (KH > 1)
+    if (!few) return launch_rows_r<KH, KW, 4>(p, co, st);
+  return launch_rows_r<KH, KW, 2>(p, co, st);
+}
+
+// `rpt` output rows per thread.
+template <int KH, int KW, int CO>
+nk_status launch_stream_co(const Direct& p, int rpt, cudaStream_t st) {
+  dim3 grid((unsigned)((p.OW + 511) / 512), (unsigned)((p.OH + rpt - 1) / rpt), (unsigned)(p.N * ((p.CO + CO - 1) / CO)));
+  if (p.beta == 0.f && !p.relu) (void)nk::launch_k(direct_stream_kernel<KH, KW, CO, true>, grid, dim3(128), 0, st, 1, p, rpt);
+  else (void)nk::launch_k(direct_stream_kernel<KH, KW, CO, false>, grid, dim3(128), 0, st, 1, p, rpt);
+  return check_launch("direct_stream_kernel");
+}
+
+// Stride 1, dilation 1, no program.  One input channel streams rows, except for
+// 5 x 5 filters (their five accumulator rows and taps fill the registers: 16 x
+// 1000 x 1000 1 -> 4, 198 us streaming, 108 by blocks of rows), 1 x 1 filters
+// with several outputs (16 x 1000 x 1001 1 -> 4: 66 / 56; 1 -> 1: 22 / 25), and
+// where a stream of four rows would give fewer than six CTAs per SM (2 x 300 x
+// 300 1 -> 4, 3 x 3: 6.5 / 3.2).  Streams are short enough that the grid walks
+// the images nearly in order, long enough to amortise the KH - 1 halo rows; us
+// for 4 / 8 / 16 rows of 16 x 1000 x 1002 1 -> 4, 3 x 3: 64 / 56 / 58.
+template <int KH, int KW>
+nk_status launch_registers(const Direct& p, cudaStream_t st) {
+  int sms = 152;
+  nk_status s = require_device(&sms);
+  if (s != NK_OK) return s;
+  const int groups = (p.CO + 3) / 4;
+  if ((int64_t)p.N * groups > 65535) return fail(NK_ERR_UNSUPPORTED, "batch x channel groups too large");
+  if ((p.OH - 1) / (p.CI == 1 ? 64 : 4) >= 65535) return fail(NK_ERR_UNSUPPORTED, "output too tall");
+  if constexpr (KH < 5) {
+    if (p.CI == 1 && (KH == 3 || p.CO == 1)) {
+      const int64_t ctas_per_row = (int64_t)((p.OW + 511) / 512) * p.N * groups;
+      constexpr int64_t kRows = KH == 1 ? 4 : 8;
+      int64_t rpt = (int64_t)p.OH * ctas_per_row / ((int64_t)sms * 6);
+      if (rpt >= 4) {
+        rpt = rpt > kRows ? kRows : rpt;
+        if ((p.OH + rpt - 1) / rpt > 65535) rpt = 64;   // grid.y
+        if constexpr (KH == 1) return launch_stream_co<KH, KW, 1>(p, (int)rpt, st);
+        else switch (p.CO) {
+          case 1: return launch_stream_co<KH, KW, 1>(p, (int)rpt, st);
+          case 2: return launch_stream_co<KH, KW, 2>(p, (int)rpt, st);
+          case 3: return launch_stream_co<KH, KW, 3>(p, (int)rpt, st);
+          default: return launch_stream_co<KH, KW, 4>(p, (int)rpt, st);
+        }
+      }
+    }
   }
+  return launch_rows<KH, KW>(p, sms, st);
 }
 
 }  // namespace
@@ -531,15 +533,10 @@ extern "C" nk_status nk_conv2d_nchw_fchw(const nk_tensor* I, const nk_tensor* K,
   // their loops would slow the plain path); a program goes to the general
   // kernel below.
   const bool plain = p.ew.n == 0;
-  if (plain && p.sh == 1 && p.sw == 1 && p.dh == 1 && p.dw == 1 && p.CI == 1) {
-    if (p.KH == 3 && p.KW == 3) return launch_stream<3, 3>(p, st);
-    if (p.KH == 5 && p.KW == 5) return launch_stream<5, 5>(p, st);
-    if (p.KH == 1 && p.KW == 1) return launch_stream<1, 1>(p, st);
-  }
   if (plain && p.sh == 1 && p.sw == 1 && p.dh == 1 && p.dw == 1) {
-    if (p.KH == 3 && p.KW == 3) return launch_rows<3, 3>(p, st);
-    if (p.KH == 5 && p.KW == 5) return launch_rows<5, 5>(p, st);
-    if (p.KH == 1 && p.KW == 1) return launch_rows<1, 1>(p, st);
+    if (p.KH == 3 && p.KW == 3) return launch_registers<3, 3>(p, st);
+    if (p.KH == 5 && p.KW == 5) return launch_registers<5, 5>(p, st);
+    if (p.KH == 1 && p.KW == 1) return launch_registers<1, 1>(p, st);
   }
   const int groups = (p.CO + CO_G - 1) / CO_G;
   if ((int64_t)p.N * groups > 65535) return fail(NK_ERR_UNSUPPORTED, "batch x channel groups too large");
