@@ -52,7 +52,10 @@ typedef struct {
 nk_status nk_enumerate_schedules(const nk_problem* p, nk_schedule* out, int32_t cap,
                                  int32_t* count);
 
-/* The built-in schedule (used when nk_matmul / nk_conv2d get sched = NULL). */
+/* The built-in schedule (used when nk_matmul / nk_conv2d get sched = NULL,
+ * but for two kinds of nk_matmul that a problem does not tell apart: an
+ * elementwise program after a short K takes 128 x 256 tiles instead of wide
+ * pairs, and BF16x3 takes wide pairs where its two-MMA steps gain by them). */
 nk_status nk_default_schedule(const nk_problem* p, nk_schedule* out);
 
 /* Workspace bytes the call for this problem needs at its precision and
