@@ -440,8 +440,10 @@ const char* nk_last_error(void);
  * cleared), NK_ERR_CUDA for a runtime error.                                */
 nk_status nk_sync_status(void* stream);
 
-/* Test hook: the spin budget (iterations) of every bounded device wait;
- * 0 restores the default.  Lets a test drive the timeout path on purpose. */
+/* Test hook: the most polls a bounded device wait makes; 0 restores the
+ * default.  Lets a test drive the timeout path on purpose: the first poll never
+ * sleeps, so with a budget of 1 every wait on a copy or an MMA that is still
+ * under way gives up, however short the kernel is.                          */
 nk_status nk_set_wait_budget(int64_t iterations);
 
 /* Programmatic dependent launch (on by default).  When on, every compute

@@ -49,18 +49,34 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait on phase `parity` of barrier `bar`.  Returns false when the
-// CTA is aborting (flag already set by another role, or this wait ran out of
-// its iteration budget or of about four seconds).  The fast path is a bare
-// poll: the wall clock (a slow register to read) and the abort flag are only
-// consulted every 1024 polls, so a wait that ends soon costs no timer read.
+// One poll that never suspends the thread.
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// Bounded wait on phase `parity` of barrier `bar`: at most `budget` polls.
+// Returns false when the CTA is aborting (flag already set by another role, or
+// this wait ran out of its polls or of about four seconds).  The first poll
+// is a test; the others may sleep in hardware, for a time nothing specifies, so
+// only a budget of one poll says how soon a wait gives up: before any copy
+// or MMA can have ended.  The wall clock (a slow register to read) and the
+// abort flag are only consulted every 1024 polls, so a wait that ends soon
+// costs no timer read.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int64_t budget,
                                           volatile int* abort_flag, unsigned int* err_word) {
+  if (mbar_test_wait(bar, parity)) return true;
   uint64_t t0 = 0;
-  for (int64_t i = 0;; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
+  for (int64_t i = 1;; ++i) {
     bool give_up = i >= budget;
-    if ((i & 1023) == 1023) {
+    if ((i & 1023) == 0) {
       if (*abort_flag) return false;
       const uint64_t now = globaltimer();
       if (t0 == 0) t0 = now;
@@ -72,6 +88,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int64_t
       __threadfence_block();
       return false;
     }
+    if (mbar_try_wait(bar, parity)) return true;
   }
 }
 
