@@ -270,12 +270,12 @@ __device__ __forceinline__ void add_bias32(const float* bias, float (&v)[32]) {
   if ((reinterpret_cast<uintptr_t>(bias) & 15) == 0) {
 #pragma unroll
     for (int j = 0; j < 32; j += 4) {
-      const float4 b = __ldg(reinterpret_cast<const float4*>(bias + j));
+      const float4 b = *reinterpret_cast<const float4*>(bias + j);
       v[j] += b.x; v[j + 1] += b.y; v[j + 2] += b.z; v[j + 3] += b.w;
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] += __ldg(bias + j);
+    for (int j = 0; j < 32; ++j) v[j] += bias[j];
   }
 }
 

@@ -80,6 +80,10 @@ __global__ void __launch_bounds__(THREADS) direct_conv_kernel(const __grid_const
   for (int ci = 0; ci < p.CI; ++ci) {
     __syncthreads();
     const float* src = p.I + n * p.sIn + ci * p.sIc;
+    for (int e = threadIdx.x; e < ncog * taps; e += THREADS) {
+      const int c = e / taps, t = e % taps;
+      ker[c * 64 + t] = p.Kr[((int64_t)(co0 + c) * p.CI + ci) * taps + t];
+    }
     // Eight loads in flight per thread before any lands in shared memory.
     const int total = p.in_h * p.in_w;
     for (int e0 = threadIdx.x; e0 < total; e0 += 8 * THREADS) {
@@ -89,15 +93,11 @@ __global__ void __launch_bounds__(THREADS) direct_conv_kernel(const __grid_const
         const int e = e0 + u * THREADS;
         const int r = e / p.in_w, c = e - r * p.in_w;
         const int ih = ih0 + r, iw = iw0 + c;
-        v[u] = (e < total && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W) ? __ldg(src + ih * p.sIh + iw) : 0.f;
+        v[u] = (e < total && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W) ? src[ih * p.sIh + iw] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         if (e0 + u * THREADS < total) tile[e0 + u * THREADS] = v[u];
-    }
-    for (int e = threadIdx.x; e < ncog * taps; e += THREADS) {
-      const int c = e / taps, t = e % taps;
-      ker[c * 64 + t] = __ldg(p.Kr + ((int64_t)(co0 + c) * p.CI + ci) * taps + t);
     }
     __syncthreads();
     for (int ki = 0; ki < p.KH; ++ki) {
@@ -150,18 +150,18 @@ __global__ void __launch_bounds__(THREADS) direct_conv_kernel(const __grid_const
 template <int SEG>
 __device__ __forceinline__ void load_row(const float* src, bool vec, int wi, int W, float (&x)[SEG]) {
   if (SEG >= 4 && vec) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(src));
+    const float4 v = *reinterpret_cast<const float4*>(src);
     x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
     if constexpr (SEG == 6) {
-      const float2 t = __ldg(reinterpret_cast<const float2*>(src + 4));
+      const float2 t = *reinterpret_cast<const float2*>(src + 4);
       x[4] = t.x; x[5] = t.y;
     } else if constexpr (SEG == 8) {
-      const float4 t = __ldg(reinterpret_cast<const float4*>(src + 4));
+      const float4 t = *reinterpret_cast<const float4*>(src + 4);
       x[4] = t.x; x[5] = t.y; x[6] = t.z; x[7] = t.w;
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < SEG; ++j) x[j] = (unsigned)(wi + j) < (unsigned)W ? __ldg(src + j) : 0.f;
+    for (int j = 0; j < SEG; ++j) x[j] = (unsigned)(wi + j) < (unsigned)W ? src[j] : 0.f;
   }
 }
 
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(128, rows_ctas(KH, CO)) direct_rows_kernel(con
     for (int c = 0; c < CO; ++c)
 #pragma unroll
       for (int t = 0; t < TAPS; ++t)
-        w[c][t] = c < ncog ? __ldg(p.Kr + ((int64_t)(co0 + c) * p.CI + ci) * TAPS + t) : 0.f;
+        w[c][t] = c < ncog ? p.Kr[((int64_t)(co0 + c) * p.CI + ci) * TAPS + t] : 0.f;
 #pragma unroll
     for (int r = 0; r < ROWS + KH - 1; ++r) {   // input row ho0 + r - pt
       float x[SEG];
@@ -269,6 +269,9 @@ __global__ void __launch_bounds__(128, rows_ctas(KH, CO)) direct_rows_kernel(con
   float* dst = p.O + n * p.sOn + (int64_t)co0 * p.sOc + (int64_t)ho0 * p.sOh + wo;
   // floats into a 16-byte word at which a row starts: wo is a multiple of 4
   const int at = (int)((reinterpret_cast<uintptr_t>(p.O) >> 2) + n * p.sOn + co0 * p.sOc + ho0 * p.sOh);
+  float bias[CO];   // read before the first store, which the compiler cannot move it across
+#pragma unroll
+  for (int c = 0; c < CO; ++c) bias[c] = (p.bias && c < ncog) ? p.bias[co0 + c] : 0.f;
 #pragma unroll
   for (int r = 0; r < ROWS; ++r) {
     if (ho0 + r >= p.OH) break;
@@ -276,7 +279,7 @@ __global__ void __launch_bounds__(128, rows_ctas(KH, CO)) direct_rows_kernel(con
     for (int c = 0; c < CO; ++c) {
       if (c >= ncog) break;
       const int s = -(at + c * (int)(p.sOc & 3) + r * (int)(p.sOh & 3)) & 3;
-      finish_row<PLAIN>(p, dst + c * p.sOc + r * p.sOh, s, full, wo, p.bias ? __ldg(p.bias + co0 + c) : 0.f, acc[r][c]);
+      finish_row<PLAIN>(p, dst + c * p.sOc + r * p.sOh, s, full, wo, bias[c], acc[r][c]);
     }
   }
 }
@@ -313,10 +316,10 @@ __global__ void __launch_bounds__(128) direct_stream_kernel(const __grid_constan
 #pragma unroll
   for (int c = 0; c < CO; ++c)
 #pragma unroll
-    for (int t = 0; t < TAPS; ++t) w[c][t] = c < ncog ? __ldg(p.Kr + (int64_t)(co0 + c) * TAPS + t) : 0.f;
+    for (int t = 0; t < TAPS; ++t) w[c][t] = c < ncog ? p.Kr[(int64_t)(co0 + c) * TAPS + t] : 0.f;
   float bias[CO];
 #pragma unroll
-  for (int c = 0; c < CO; ++c) bias[c] = (p.bias && c < ncog) ? __ldg(p.bias + co0 + c) : 0.f;
+  for (int c = 0; c < CO; ++c) bias[c] = (p.bias && c < ncog) ? p.bias[co0 + c] : 0.f;
   // Accumulators of the KH output rows under way.  A row's first tap row
   // overwrites its slot, so the rows above the first output row (o < 0) leave
   // nothing behind, and those past the last are never stored.

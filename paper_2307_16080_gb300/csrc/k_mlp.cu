@@ -49,25 +49,23 @@ struct Smem {
   float sq[ROWS];
 };
 
-__device__ void load_weights(const float* __restrict__ P, Smem& s) {
+__device__ void load_weights(const float* P, Smem& s) {
   const int t = threadIdx.x;
 #pragma unroll 8
-  for (int e = t; e < D1 * D2; e += THREADS) s.w2t[e % D1][e / D1] = __ldg(P + OFF_W2 + e);
+  for (int e = t; e < D1 * D2; e += THREADS) s.w2t[e % D1][e / D1] = P[OFF_W2 + e];
 #pragma unroll
-  for (int e = t; e < D1 * D0; e += THREADS) s.w1[e / D0][e % D0] = __ldg(P + OFF_W1 + e);
+  for (int e = t; e < D1 * D0; e += THREADS) s.w1[e / D0][e % D0] = P[OFF_W1 + e];
 }
 
 // Forward for rows r0 .. r0 + 7; fills s.x, z1, h1, h1t, z2.  y[q] of the
 // thread's four rows is h2 * W3 of its hidden unit, and the row's output is
 // the sum over s.part[row] plus b3.  Ends with the sums in place.
-__device__ __forceinline__ void forward_rows(const float* __restrict__ X, int64_t B, int64_t r0, float b1, float b2,
+__device__ __forceinline__ void forward_rows(const float* X, int64_t B, int64_t r0, float b1, float b2,
                                              float w3, Smem& s, float (&h2)[4]) {
   const int t = threadIdx.x, j = t & 127, rq = (t >> 7) * 4;
+  const float xv = t < ROWS * D0 && r0 + t / D0 < B ? X[r0 * D0 + t] : 0.f;   // under way across the barrier
   __syncthreads();   // the step before has read everything (first step: the weights are in)
-  if (t < ROWS * D0) {
-    const int r = t / D0;
-    s.x[r][t % D0] = (r0 + r < B) ? __ldg(X + (r0 + r) * D0 + t % D0) : 0.f;
-  }
+  if (t < ROWS * D0) s.x[t / D0][t % D0] = xv;
   __syncthreads();
   float h[4];
 #pragma unroll
@@ -107,8 +105,7 @@ __device__ __forceinline__ float row_output(const Smem& s, int r, float b3) {
   return ((s.part[r][0] + s.part[r][1]) + (s.part[r][2] + s.part[r][3])) + b3;
 }
 
-__global__ void __launch_bounds__(THREADS) mlp_forward_kernel(const float* __restrict__ P,
-                                                              const float* __restrict__ X, int64_t B,
+__global__ void __launch_bounds__(THREADS) mlp_forward_kernel(const float* P, const float* X, int64_t B,
                                                               float* __restrict__ y) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
@@ -116,7 +113,7 @@ __global__ void __launch_bounds__(THREADS) mlp_forward_kernel(const float* __res
   Smem& s = *reinterpret_cast<Smem*>(raw);
   const int t = threadIdx.x, j = t & 127;
   load_weights(P, s);
-  const float b1 = __ldg(P + OFF_B1 + j), b2 = __ldg(P + OFF_B2 + j), w3 = __ldg(P + OFF_W3 + j), b3 = __ldg(P + OFF_B3);
+  const float b1 = P[OFF_B1 + j], b2 = P[OFF_B2 + j], w3 = P[OFF_W3 + j], b3 = P[OFF_B3];
   for (int64_t r0 = (int64_t)blockIdx.x * ROWS; r0 < B; r0 += (int64_t)gridDim.x * ROWS) {
     float h2[4];
     forward_rows(X, B, r0, b1, b2, w3, s, h2);
@@ -132,9 +129,7 @@ __global__ void __launch_bounds__(THREADS) mlp_forward_kernel(const float* __res
 // latency bounds it: 8-row steps give a batch of 1024 128 blocks of eight
 // warps, where 32-row blocks gave 32 of four with serial loops over rows and
 // units.  A training step (gradient, reduce, Adam) on 1024 rows: 102 -> 21 us.
-__global__ void __launch_bounds__(THREADS) mlp_grad_kernel(const float* __restrict__ P,
-                                                           const float* __restrict__ X,
-                                                           const float* __restrict__ T, int64_t B,
+__global__ void __launch_bounds__(THREADS) mlp_grad_kernel(const float* P, const float* X, const float* T, int64_t B,
                                                            float* __restrict__ part) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
@@ -143,7 +138,7 @@ __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(const float* __restri
   const int t = threadIdx.x, j = t & 127, half = t >> 7, rq = half * 4;
   const int jt = (t >> 4) * 8, it = (t & 15) * 4;   // W2 block of this thread: rows jt.., columns it.. and 64 + it..
   load_weights(P, s);
-  const float b1 = __ldg(P + OFF_B1 + j), b2 = __ldg(P + OFF_B2 + j), w3 = __ldg(P + OFF_W3 + j), b3 = __ldg(P + OFF_B3);
+  const float b1 = P[OFF_B1 + j], b2 = P[OFF_B2 + j], w3 = P[OFF_W3 + j], b3 = P[OFF_B3];
   const float inv2b = 2.f / (float)B;
   float gw2[8][8], gw1[D0 / 2];
 #pragma unroll
@@ -155,10 +150,11 @@ __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(const float* __restri
   float gw3 = 0.f, gb2 = 0.f, gb1 = 0.f, gb3 = 0.f, gsq = 0.f;
   for (int64_t r0 = (int64_t)blockIdx.x * ROWS; r0 < B; r0 += (int64_t)gridDim.x * ROWS) {
     float h2[4];
+    const bool ok = t < ROWS && r0 + t < B;
+    const float target = ok ? T[r0 + t] : 0.f;
     forward_rows(X, B, r0, b1, b2, w3, s, h2);
     if (t < ROWS) {
-      const bool ok = r0 + t < B;
-      const float d = ok ? row_output(s, t, b3) - __ldg(T + r0 + t) : 0.f;
+      const float d = ok ? row_output(s, t, b3) - target : 0.f;
       s.dy[t] = inv2b * d;
       s.sq[t] = d * d;
     }
@@ -246,7 +242,7 @@ __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(const float* __restri
 // a parameter sum every fourth block in order and are added in a fixed tree,
 // so the result is the same every run; sixteen loads in flight a thread.
 constexpr int RED_P = 64;
-__global__ void __launch_bounds__(4 * RED_P) mlp_reduce_kernel(const float* __restrict__ part, int nblocks, int64_t B,
+__global__ void __launch_bounds__(4 * RED_P) mlp_reduce_kernel(const float* part, int nblocks, int64_t B,
                                                                float* __restrict__ grad, float* __restrict__ loss) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
@@ -256,7 +252,7 @@ __global__ void __launch_bounds__(4 * RED_P) mlp_reduce_kernel(const float* __re
   float a = 0.f;
   if (p <= NPARAM) {
 #pragma unroll 16
-    for (int b = q; b < nblocks; b += 4) a += __ldg(part + (int64_t)b * (NPARAM + 1) + p);
+    for (int b = q; b < nblocks; b += 4) a += part[(int64_t)b * (NPARAM + 1) + p];
   }
   sm[q][lp] = a;
   __syncthreads();
@@ -266,7 +262,7 @@ __global__ void __launch_bounds__(4 * RED_P) mlp_reduce_kernel(const float* __re
   else if (loss) *loss = a / (float)B;
 }
 
-__global__ void mlp_adam_kernel(float* __restrict__ P, const float* __restrict__ g, float* __restrict__ m,
+__global__ void mlp_adam_kernel(float* __restrict__ P, const float* g, float* __restrict__ m,
                                 float* __restrict__ v, int n, float lr, float b1, float b2, float eps,
                                 float bc1, float bc2) {
   nk::pdl_wait();      // earlier kernels on the stream have finished

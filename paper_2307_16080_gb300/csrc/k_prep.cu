@@ -44,9 +44,12 @@ __device__ __forceinline__ void pro4(const EwProg& e, float* v, int64_t off) {
 // per block; stage 2: one block folds the partials.  NaN inputs make the
 // result NaN (the scale then falls back to 1).  PRO: the amax of the values
 // after the prologue program `pro`.
+// Registers for five blocks an SM: four (52 registers) take 43.9 us instead of
+// 39.8 for 268 MB.
 template <bool PRO>
-__global__ void amax_stage1(const float* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
-                            float* __restrict__ partial, const __grid_constant__ EwProg pro) {
+__global__ void __launch_bounds__(256, PRO ? 2 : 5) amax_stage1(const float* x, int64_t rows, int64_t cols, int64_t ld,
+                                                                float* __restrict__ partial,
+                                                                const __grid_constant__ EwProg pro) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
   float m = 0.f;
@@ -71,11 +74,11 @@ __global__ void amax_stage1(const float* __restrict__ x, int64_t rows, int64_t c
     for (; i + 7 * stride < n4; i += 8 * stride) {
       float4 v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = __ldg(x4 + i + u * stride);
+      for (int u = 0; u < 8; ++u) v[u] = x4[i + u * stride];
 #pragma unroll
       for (int u = 0; u < 8; ++u) fold(v[u], i + u * stride);
     }
-    for (; i < n4; i += stride) fold(__ldg(x4 + i), i);
+    for (; i < n4; i += stride) fold(x4[i], i);
   } else {
     // strided rows: blocks stride over rows, threads over the row
     const bool vec = al && (cols % 4 == 0) && (ld % 4 == 0);
@@ -83,7 +86,7 @@ __global__ void amax_stage1(const float* __restrict__ x, int64_t rows, int64_t c
       const float* row = x + r * ld;
       if (vec) {
         for (int64_t c = threadIdx.x; c < cols / 4; c += blockDim.x) {
-          float4 v = __ldg(reinterpret_cast<const float4*>(row) + c);
+          float4 v = reinterpret_cast<const float4*>(row)[c];
           if constexpr (PRO) {
             float w[4] = {v.x, v.y, v.z, v.w};
             pro4<PRO>(pro, w, r * ld + 4 * c);
@@ -117,7 +120,7 @@ __global__ void amax_stage1(const float* __restrict__ x, int64_t rows, int64_t c
   }
 }
 
-__global__ void amax_stage2(const float* __restrict__ partial, int n, float* __restrict__ out) {
+__global__ void amax_stage2(const float* partial, int n, float* __restrict__ out) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
   float m = 0.f;
@@ -181,8 +184,8 @@ struct Caster<2> {
 // x 1999 (48 MB), now 10.5; BF16 of 8192^2 (402 MB) 64 us, now 54.
 // PRO: the prologue program `pro` runs on each element before the cast.
 template <int KIND, bool PRO>
-__global__ void __launch_bounds__(256) cast_rows(const float* __restrict__ in, int64_t rows, int64_t cols, int64_t ld_in,
-                                                 const float* __restrict__ amax, typename Caster<KIND>::T* __restrict__ o0,
+__global__ void __launch_bounds__(256) cast_rows(const float* in, int64_t rows, int64_t cols, int64_t ld_in,
+                                                 const float* amax, typename Caster<KIND>::T* __restrict__ o0,
                                                  typename Caster<KIND>::T* __restrict__ o1, int64_t ld_out,
                                                  float* scale_out, int tx_log, const __grid_constant__ EwProg pro) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
@@ -203,12 +206,12 @@ __global__ void __launch_bounds__(256) cast_rows(const float* __restrict__ in, i
     const float* src = in + r * ld_in + c;
     float v[V];
     if (vin) {
-      const float4 q0 = __ldg(reinterpret_cast<const float4*>(src)), q1 = __ldg(reinterpret_cast<const float4*>(src + 4));
+      const float4 q0 = *reinterpret_cast<const float4*>(src), q1 = *reinterpret_cast<const float4*>(src + 4);
       v[0] = q0.x; v[1] = q0.y; v[2] = q0.z; v[3] = q0.w;
       v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
     } else {
 #pragma unroll
-      for (int j = 0; j < V; ++j) v[j] = c + j < cols ? __ldg(src + j) : 0.f;
+      for (int j = 0; j < V; ++j) v[j] = c + j < cols ? src[j] : 0.f;
     }
     if constexpr (PRO) {
 #pragma unroll
@@ -248,8 +251,8 @@ __global__ void __launch_bounds__(256) cast_rows(const float* __restrict__ in, i
 // neither side has a bank conflict.  HBM-bound: 8192^2 to BF16 (402 MB) 70 us
 // with an FP32 tile and two-way conflicts, now 53.
 template <int KIND, bool PRO>
-__global__ void __launch_bounds__(256) cast_transpose(const float* __restrict__ in, int64_t rows, int64_t cols,
-                                                      int64_t ld_in, const float* __restrict__ amax,
+__global__ void __launch_bounds__(256) cast_transpose(const float* in, int64_t rows, int64_t cols,
+                                                      int64_t ld_in, const float* amax,
                                                       typename Caster<KIND>::T* __restrict__ o0,
                                                       typename Caster<KIND>::T* __restrict__ o1, int64_t ld_out,
                                                       float* scale_out, const __grid_constant__ EwProg pro) {
@@ -276,12 +279,12 @@ __global__ void __launch_bounds__(256) cast_transpose(const float* __restrict__ 
       x[0] = x[1] = x[2] = x[3] = 0.f;
       if (r < rows) {
         if (vin) {
-          const float4 q = __ldg(reinterpret_cast<const float4*>(in + r * ld_in + c));
+          const float4 q = *reinterpret_cast<const float4*>(in + r * ld_in + c);
           x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
         } else {
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            if (c + j < cols) x[j] = __ldg(in + r * ld_in + c + j);
+            if (c + j < cols) x[j] = in[r * ld_in + c + j];
         }
       }
     }
@@ -345,7 +348,7 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 
 // Fixed-order FP64 block sums: thread i of block b visits elements
 // b*blockDim + i + k*gridDim*blockDim; warp tree, then a tree over warps.
-__global__ void norm_stage1(const float* __restrict__ C, int64_t ldc, const double* __restrict__ R,
+__global__ void norm_stage1(const float* C, int64_t ldc, const double* R,
                             int64_t ldr, int64_t M, int64_t N, double* __restrict__ partial) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
@@ -374,7 +377,7 @@ __global__ void norm_stage1(const float* __restrict__ C, int64_t ldc, const doub
   }
 }
 
-__global__ void norm_stage2(const double* __restrict__ partial, int n, double* __restrict__ out) {
+__global__ void norm_stage2(const double* partial, int n, double* __restrict__ out) {
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
   double e = 0.0, r2 = 0.0;

@@ -99,7 +99,7 @@ __device__ __forceinline__ void finish4(const SimtGemm& p, int m, int nb, const 
     float o = p.alpha * acc[j];
     if (n < p.N) {
       if (p.beta != 0.f) o = fmaf(p.beta, crow[(int64_t)n * p.scn], o);
-      if (p.bias) o += __ldg(p.bias + (p.bias_on_m ? m : n));
+      if (p.bias) o += p.bias[p.bias_on_m ? m : n];
       if (p.relu) o = (o > 0.f || o != o) ? o : 0.f;
     }
     v[j] = o;
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(256) splitk_reduce4_kernel(const __grid_consta
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (s < r.splits) q = __ldg(reinterpret_cast<const float4*>(r.partial + s * slice + (int64_t)m * r.ldp + n));
+      if (s < r.splits) q = *reinterpret_cast<const float4*>(r.partial + s * slice + (int64_t)m * r.ldp + n);
       v[s][0] = q.x; v[s][1] = q.y; v[s][2] = q.z; v[s][3] = q.w;
     }
 #pragma unroll
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(256) splitk_reduce4_kernel(const __grid_consta
       o[e] = alpha * v[0][e];
       if (n + e >= r.N) continue;
       if (r.beta != 0.f) o[e] = fmaf(r.beta, r.out_bf16 ? __bfloat162float(ch[e]) : c[e], o[e]);
-      if (r.bias) o[e] += __ldg(r.bias + (r.bias_on_m ? m : n + e));
+      if (r.bias) o[e] += r.bias[r.bias_on_m ? m : n + e];
       if (r.relu) o[e] = (o[e] > 0.f || o[e] != o[e]) ? o[e] : 0.f;
     }
     if (word && r.out_bf16) {

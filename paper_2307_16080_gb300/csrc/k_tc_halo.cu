@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
               const float4* tr = reinterpret_cast<const float4*>(p.ew.t[0] + orow_off + col0);
 #pragma unroll
               for (int j = 0; j < 32; j += 4) {
-                const float4 r4 = __ldg(tr + j / 4);
+                const float4 r4 = tr[j / 4];
                 const float rv[4] = {r4.x, r4.y, r4.z, r4.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
                 float xv = v[j];
                 if (j < ncol) {
                   if (p.beta != 0.f) xv = fmaf(p.beta, __bfloat162float(dh[j]), xv);
-                  if (p.bias) xv += __ldg(p.bias + col0 + j);
+                  if (p.bias) xv += p.bias[col0 + j];
                   if (p.relu) xv = (xv > 0.f || xv != xv) ? xv : 0.f;
                 }
                 buf[j] = xv;
@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
                 float xv = v[j];
                 if (col0 + j < p.F) {
                   if (p.beta != 0.f) xv = fmaf(p.beta, __bfloat162float(dh[j]), xv);
-                  if (p.bias) xv += __ldg(p.bias + col0 + j);
+                  if (p.bias) xv += p.bias[col0 + j];
                   if (p.relu) xv = (xv > 0.f || xv != xv) ? xv : 0.f;
                 }
                 v[j] = xv;
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
               float xv = v[j];
               if (j < ncol) {
                 if (p.beta != 0.f) xv = fmaf(p.beta, dst[j], xv);
-                if (p.bias) xv += __ldg(p.bias + col0 + j);
+                if (p.bias) xv += p.bias[col0 + j];
                 if (p.relu) xv = (xv > 0.f || xv != xv) ? xv : 0.f;
               }
               buf[j] = xv;
@@ -526,35 +526,41 @@ __global__ void __launch_bounds__(DB ? kThreadsDB : kThreads, 1) halo_conv_kerne
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
               float xv = v[j];
-              if (p.bias) xv += __ldg(p.bias + col0 + j);
+              if (p.bias) xv += p.bias[col0 + j];
               if (p.relu) xv = (xv > 0.f || xv != xv) ? xv : 0.f;
               v[j] = xv;
             }
             store32_f32_v8(dst, v);
           } else if (p.c_vec && col0 + 32 <= p.F) {
+            // all loads before the first store (the compiler cannot know that O
+            // aliases no bias)
+            if (p.beta != 0.f) {
+              float4 cin[8];
 #pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-              float o[4];
-              float4 cin = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (p.beta != 0.f) cin = *reinterpret_cast<const float4*>(dst + j);
-              const float ci[4] = {cin.x, cin.y, cin.z, cin.w};
+              for (int j = 0; j < 8; ++j) cin[j] = *reinterpret_cast<const float4*>(dst + 4 * j);
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                float xv = v[j + e];
-                if (p.beta != 0.f) xv = fmaf(p.beta, ci[e], xv);
-                if (p.bias) xv += __ldg(p.bias + col0 + j + e);
-                if (p.relu) xv = (xv > 0.f || xv != xv) ? xv : 0.f;
-                o[e] = xv;
+              for (int j = 0; j < 32; j += 4) {
+                v[j] = fmaf(p.beta, cin[j / 4].x, v[j]);
+                v[j + 1] = fmaf(p.beta, cin[j / 4].y, v[j + 1]);
+                v[j + 2] = fmaf(p.beta, cin[j / 4].z, v[j + 2]);
+                v[j + 3] = fmaf(p.beta, cin[j / 4].w, v[j + 3]);
               }
-              *reinterpret_cast<float4*>(dst + j) = make_float4(o[0], o[1], o[2], o[3]);
             }
+            if (p.bias) add_bias32(p.bias + col0, v);
+            if (p.relu) {
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] = (v[j] > 0.f || v[j] != v[j]) ? v[j] : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 32; j += 4)
+              *reinterpret_cast<float4*>(dst + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
           } else {
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
               if (col0 + j >= p.F) continue;
               float xv = v[j];
               if (p.beta != 0.f) xv = fmaf(p.beta, dst[j], xv);
-              if (p.bias) xv += __ldg(p.bias + col0 + j);
+              if (p.bias) xv += p.bias[col0 + j];
               if (p.relu) xv = (xv > 0.f || xv != xv) ? xv : 0.f;
               dst[j] = xv;
             }

@@ -60,6 +60,14 @@ int64_t wait_budget();
 // and needs nothing from the later one, so a later CTA blocked in pdl_wait()
 // or in a TMEM allocation cannot hold it up.  Launched without the attribute
 // (nk_set_pdl(0)) both instructions do nothing.
+//
+// What an earlier kernel may have written -- every operand, bias, partial sum
+// and scale -- is read with plain loads.  A non-coherent load (__ldg, or a
+// const __restrict__ parameter of a kernel, which the compiler may turn into
+// one) is for data that nobody writes while the grid runs, and a grid that was
+// started early runs while its predecessor still writes: such a load may also
+// move ahead of pdl_wait().  Only a plan's own tables, which the host filled
+// before any launch, are read that way.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -571,7 +571,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
           const int col_begin = t.tn * p.bn + c_begin;
           const int nseg = max(0, min(c_cols, t.N - col_begin) + 31) / 32;
           const uint32_t ta0 = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * acc_cols + c_begin);
-          const float bm = (t.bias && p.bias_on_m && row_ok) ? __ldg(t.bias + row) : 0.f;
+          const float bm = (t.bias && p.bias_on_m && row_ok) ? t.bias[row] : 0.f;
           constexpr int PARTS = KIND == TC_BF16X3 ? 2 : 1;
           constexpr int AHEAD = 2 / PARTS;   // segments whose TMEM loads share one wait
           auto load = [&](int i, uint32_t (&r)[PARTS][32]) {
@@ -594,12 +594,12 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
               } else if (col0 + 32 <= t.N && (reinterpret_cast<uintptr_t>(t.bias + col0) & 15) == 0) {
 #pragma unroll
                 for (int j = 0; j < 32; j += 4) {
-                  const float4 b = __ldg(reinterpret_cast<const float4*>(t.bias + col0 + j));
+                  const float4 b = *reinterpret_cast<const float4*>(t.bias + col0 + j);
                   v[j] += b.x; v[j + 1] += b.y; v[j + 2] += b.z; v[j + 3] += b.w;
                 }
               } else {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] += col0 + j < t.N ? __ldg(t.bias + col0 + j) : 0.f;
+                for (int j = 0; j < 32; ++j) v[j] += col0 + j < t.N ? t.bias[col0 + j] : 0.f;
               }
             }
             if (t.relu) {
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
               const float4* tr = reinterpret_cast<const float4*>(p.ew.t[0] + off);
 #pragma unroll
               for (int j = 0; j < 32; j += 4) {
-                const float4 r4 = __ldg(tr + j / 4);
+                const float4 r4 = tr[j / 4];
                 const float rv[4] = {r4.x, r4.y, r4.z, r4.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -745,7 +745,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
               float x = alpha * v[j];
               if (j < ncol) {
                 if (t.beta != 0.f) x = fmaf(t.beta, __bfloat162float(dh[j]), x);
-                if (t.bias) x += __ldg(t.bias + col0 + j);
+                if (t.bias) x += t.bias[col0 + j];
                 if (t.relu) x = (x > 0.f || x != x) ? x : 0.f;
               }
               buf[j] = x;
@@ -760,14 +760,14 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
           }
         }
         float* dst = t.C + (int64_t)row * t.ldc + col0;
-        const float bm = (t.bias && p.bias_on_m) ? __ldg(t.bias + row) : 0.f;
+        const float bm = (t.bias && p.bias_on_m) ? t.bias[row] : 0.f;
         const float beta = t.beta;
         if (!CONV && p.c_vec32 && beta == 0.f && col0 + 32 <= t.N && p.ew.n == 0) {
           // full 32-column segment of 32-byte aligned rows: 32-byte stores
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             float x = alpha * v[j];
-            if (t.bias) x += p.bias_on_m ? bm : __ldg(t.bias + col0 + j);
+            if (t.bias) x += p.bias_on_m ? bm : t.bias[col0 + j];
             if (t.relu) x = (x > 0.f || x != x) ? x : 0.f;
             v[j] = x;
           }
@@ -786,7 +786,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
             float x = alpha * v[j];
             if (j < ncol) {
               if (beta != 0.f) x = fmaf(beta, dst[j], x);
-              if (t.bias) x += p.bias_on_m ? bm : __ldg(t.bias + col0 + j);
+              if (t.bias) x += p.bias_on_m ? bm : t.bias[col0 + j];
               if (t.relu) x = (x > 0.f || x != x) ? x : 0.f;
             }
             buf[j] = x;
@@ -811,7 +811,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
             for (int e = 0; e < 4; ++e) {
               float x = alpha * v[j + e];
               if (beta != 0.f) x = fmaf(beta, ci[e], x);
-              if (t.bias) x += p.bias_on_m ? bm : __ldg(t.bias + col0 + j + e);
+              if (t.bias) x += p.bias_on_m ? bm : t.bias[col0 + j + e];
               if (t.relu) x = (x > 0.f || x != x) ? x : 0.f;
               o[e] = x;
             }
@@ -823,7 +823,7 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
             if (col0 + j >= t.N) continue;
             float x = alpha * v[j];
             if (beta != 0.f) x = fmaf(beta, dst[j], x);
-            if (t.bias) x += p.bias_on_m ? bm : __ldg(t.bias + col0 + j);
+            if (t.bias) x += p.bias_on_m ? bm : t.bias[col0 + j];
             if (t.relu) x = (x > 0.f || x != x) ? x : 0.f;
             dst[j] = x;
           }
