@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <mutex>
 
 #include "nk_internal.cuh"
@@ -41,7 +42,6 @@ struct KArgs {
   int k_chunk;      // reduction length handled by one grid-z slice
   float* partial;   // [splits][M][N] or null
   int csplit;       // CTAs of a cluster that share one tile's reduction (1: none)
-  int tiles_n;
 };
 
 // Implicit im2col element A[m,k] of the convolution (0 outside the input);
@@ -118,22 +118,29 @@ __device__ __forceinline__ void finish4(const SimtGemm& p, int m, int nb, const 
 // instruction on pairs of columns (fma.rn.f32x2, each half rounded as fmaf:
 // the sums are bitwise those of a scalar loop); operands come through a ring
 // of asynchronous copies, which need no registers, no second pass to store
-// and no alignment -- a row of odd length loads as fast as an aligned one;
-// rows past M (columns past N) read a clamped row whose results are dropped,
-// so only the end of K is predicated.  A loop of these FMAs over resident tiles
+// and no alignment -- a row of odd length loads as fast as an aligned one.
+// Rows past M and columns past N are copied as zeros, without a read, in the
+// tiles 64 wide: lanes that read one clamped address instead take turns (8192 x
+// 8 x 144, built-in tile: 23.5 us so, 7.3 now; 200 x 1500 x 700 in 64 x 64 tiles,
+// whose last tiles have 8 rows: 39.7 / 26).  4-byte copies along k clamp (16
+// lanes of a row read 16 addresses), and so does the 128 x 128 tile, which
+// narrow outputs do not take and whose registers have no room for the test
+// (1531 x 2047 x 1021: 149 / 154).  A loop of these FMAs over resident tiles
 // reaches 66 TFLOP/s (scalar FMAs 60); the kernel 56 at 4096^3 (54 before).
 // Odd row lengths, which took scalar loads: 1531 x 2047 x 1021 230 -> 150 us.
 template <int BM, int BN, int T, int AM, int BMD>
 __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __grid_constant__ KArgs args) {
   constexpr int S = 4;                  // stages
-  constexpr int TY = BM / 8, TX = T / TY, TN = BN / TX;
+  constexpr int RM = BM * BN / T >= 32 ? 8 : 4;   // rows of a thread
+  constexpr int TY = BM / RM, TX = T / TY, TN = BN / TX;
   constexpr bool CONV = AM == L_CONV || AM == L_CONV16;
   constexpr bool AMK = AM == L_CONV16 || AM == L_K16;   // A is stored [m][k]
   constexpr int A_LD = AMK ? BK + 4 : BM + 4, B_LD = BN + 4;
   constexpr int A_FL = AMK ? BM * A_LD : BK * A_LD;
   constexpr int STAGE = A_FL + BK * B_LD;
-  constexpr int KV = T == 256 ? 2 : 4;   // k values of A in registers at a time (256 threads: 128 registers each)
-  static_assert(TN == 8 || TN == 4, "8 x 8 or 8 x 4 outputs per thread");
+  constexpr bool SKIP = BN == 64;        // no reads past M and N
+  constexpr int KV = T == 256 && RM == 8 ? 2 : 4;   // k values of A in registers at a time (256 threads: 128 registers each)
+  static_assert(TN == 8 || TN == 4, "8 x 8, 8 x 4 or 4 x 4 outputs per thread");
   static_assert(S * STAGE >= BM * BN, "a cluster's partial tiles reuse the ring");
   extern __shared__ __align__(16) float smem[];
   __shared__ int row_off[BM], row_hw[BM];   // conv: offset of a row's first tap, and its (ih, iw)
@@ -158,7 +165,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
       const int ow = m % g.ow, q = m / g.ow, oh = q % g.oh, n = q / g.oh;
       const int ih = oh * g.sh - g.pt, iw = ow * g.sw - g.pl;
       row_off[r] = (int)(n * g.sin_n + ih * g.sin_h + iw * g.sin_w);
-      row_hw[r] = (ih << 16) | (iw & 0xffff);
+      row_hw[r] = m0 + r < p.M ? (ih << 16) | (iw & 0xffff) : INT_MIN;   // past the end: above every input
     }
     __syncthreads();
   }
@@ -197,27 +204,32 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
       const int k = k0 + ak;
       const bool ok = k < kend;
       const float* src = p.A + (int64_t)(ok ? k : 0) * p.sak;
+      const int rows = KC == 4 && SKIP ? p.M - m0 - ar : BM;   // this thread's rows that exist (4-byte copies clamp)
 #pragma unroll
       for (int i = 0; i < BM / AR; ++i) {
         const int r = ar + i * AR;
-        cpa(sa + (uint32_t)((AMK ? r * A_LD + ak : ak * A_LD + r) * 4), src + (int64_t)min(m0 + r, p.M - 1) * p.sam, ok);
+        cpa(sa + (uint32_t)((AMK ? r * A_LD + ak : ak * A_LD + r) * 4), src + (int64_t)min(m0 + r, p.M - 1) * p.sam,
+            ok && i * AR < rows);
       }
     } else if constexpr (AM == L_MN) {
       const int r = tid % BM;
+      const bool in = !SKIP || m0 + r < p.M;
+      const float* src = p.A + (int64_t)min(m0 + r, p.M - 1) * p.sam;
 #pragma unroll
       for (int i = 0; i < BK * BM / T; ++i) {
         const int kk = tid / BM + i * (T / BM);
         const bool ok = k0 + kk < kend;
-        cp4(sa + (uint32_t)((kk * A_LD + r) * 4),
-            p.A + (int64_t)(ok ? k0 + kk : 0) * p.sak + (int64_t)min(m0 + r, p.M - 1) * p.sam, ok);
+        cp4(sa + (uint32_t)((kk * A_LD + r) * 4), src + (int64_t)(ok ? k0 + kk : 0) * p.sak, ok && in);
       }
     } else {
       const int r = tid % (BM / 4) * 4;
+      const bool in = !SKIP || m0 + r < p.M;
+      const float* src = p.A + min(m0 + r, p.M - 4);
 #pragma unroll
       for (int i = 0; i < BK * BM / 4 / T; ++i) {
         const int kk = tid / (BM / 4) + i * (T / (BM / 4));
         const bool ok = k0 + kk < kend;
-        cp16(sa + (uint32_t)((kk * A_LD + r) * 4), p.A + (int64_t)(ok ? k0 + kk : 0) * p.sak + min(m0 + r, p.M - 4), ok);
+        cp16(sa + (uint32_t)((kk * A_LD + r) * 4), src + (int64_t)(ok ? k0 + kk : 0) * p.sak, ok && in);
       }
     }
     if constexpr (BMD == L_K) {
@@ -231,27 +243,30 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
       }
     } else if constexpr (BMD == L_MN) {
       const int c = tid % BN;
+      const bool in = !SKIP || n0 + c < p.N;
+      const float* src = p.B + (int64_t)min(n0 + c, p.N - 1) * p.sbn;
 #pragma unroll
       for (int i = 0; i < BK * BN / T; ++i) {
         const int kk = tid / BN + i * (T / BN);
         const bool ok = k0 + kk < kend;
-        cp4(sb + (uint32_t)((kk * B_LD + c) * 4),
-            p.B + (int64_t)(ok ? k0 + kk : 0) * p.sbk + (int64_t)min(n0 + c, p.N - 1) * p.sbn, ok);
+        cp4(sb + (uint32_t)((kk * B_LD + c) * 4), src + (int64_t)(ok ? k0 + kk : 0) * p.sbk, ok && in);
       }
     } else {
       const int c = tid % (BN / 4) * 4;
+      const bool in = !SKIP || n0 + c < p.N;
+      const float* src = p.B + min(n0 + c, p.N - 4);
 #pragma unroll
       for (int i = 0; i < BK * BN / 4 / T; ++i) {
         const int kk = tid / (BN / 4) + i * (T / (BN / 4));
         const bool ok = k0 + kk < kend;
-        cp16(sb + (uint32_t)((kk * B_LD + c) * 4), p.B + (int64_t)(ok ? k0 + kk : 0) * p.sbk + min(n0 + c, p.N - 4), ok);
+        cp16(sb + (uint32_t)((kk * B_LD + c) * 4), src + (int64_t)(ok ? k0 + kk : 0) * p.sbk, ok && in);
       }
     }
   };
 
-  f2 acc[8][TN / 2];
+  f2 acc[RM][TN / 2];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
     for (int j = 0; j < TN / 2; ++j) acc[i][j] = f2_set(0.f);
 
@@ -267,7 +282,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
     asm volatile("cp.async.commit_group;" ::: "memory");
     const float* As = smem + (t % S) * STAGE;
     const float* Bs = As + A_FL;
-    auto step = [&](int kk, const float (&a)[8]) {
+    auto step = [&](int kk, const float (&a)[RM]) {
       f2 b[TN / 2];
 #pragma unroll
       for (int h = 0; h < TN / 4; ++h) {
@@ -276,7 +291,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
         b[2 * h + 1].v = q.y;
       }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < RM; ++i) {
         const f2 aa = f2_set(a[i]);
 #pragma unroll
         for (int j = 0; j < TN / 2; ++j) acc[i][j] = f2_fma(aa, b[j], acc[i][j]);
@@ -285,9 +300,9 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
     if constexpr (AMK) {
 #pragma unroll
       for (int kq = 0; kq < BK; kq += KV) {
-        float av[8][KV];
+        float av[RM][KV];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < RM; ++i) {
           const float* src = As + (ty + TY * i) * A_LD + kq;
           if constexpr (KV == 4) {
             const float4 q = *reinterpret_cast<const float4*>(src);
@@ -299,18 +314,21 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
         }
 #pragma unroll
         for (int e = 0; e < KV; ++e) {
-          float a[8];
+          float a[RM];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) a[i] = av[i][e];
+          for (int i = 0; i < RM; ++i) a[i] = av[i][e];
           step(kq + e, a);
         }
       }
     } else {
 #pragma unroll
       for (int kk = 0; kk < BK; ++kk) {
-        const float4 a0 = *reinterpret_cast<const float4*>(As + kk * A_LD + ty * 4);
-        const float4 a1 = *reinterpret_cast<const float4*>(As + kk * A_LD + BM / 2 + ty * 4);
-        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        float a[RM];
+#pragma unroll
+        for (int h = 0; h < RM / 4; ++h) {
+          const float4 q = *reinterpret_cast<const float4*>(As + kk * A_LD + h * (BM / 2) + ty * 4);
+          a[4 * h] = q.x; a[4 * h + 1] = q.y; a[4 * h + 2] = q.z; a[4 * h + 3] = q.w;
+        }
         step(kk, a);
       }
     }
@@ -325,7 +343,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
       for (int h = 0; h < TN / 4; ++h) {
         const int r = row_of(i), c = h * (BN / 2) + tx * 4;
@@ -353,7 +371,7 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
   }
   // Epilogue: partial tile to the workspace, or the fused epilogue to C.
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < RM; ++i) {
     const int m = m0 + row_of(i);
     if (m >= p.M) continue;
 #pragma unroll
@@ -660,8 +678,8 @@ template <int BM, int BN, int T>
 nk_status launch_a(const KArgs& a, int amode, int bmode, dim3 grid, cudaStream_t st) {
   switch (amode) {
     case L_K: return launch_b<BM, BN, T, L_K>(a, bmode, grid, st);
-    case L_K16:   // 256 threads have no registers for [m][k] (2629 us against 2460 at 4096^3)
-      if constexpr (T == 256) return launch_b<BM, BN, T, L_K>(a, bmode, grid, st);
+    case L_K16:   // 128 x 128 tiles have no registers for [m][k] (2629 us against 2460 at 4096^3)
+      if constexpr (BN == 128) return launch_b<BM, BN, T, L_K>(a, bmode, grid, st);
       else return launch_b<BM, BN, T, L_K16>(a, bmode, grid, st);
     case L_MN: return launch_b<BM, BN, T, L_MN>(a, bmode, grid, st);
     case L_MN16: return launch_b<BM, BN, T, L_MN16>(a, bmode, grid, st);
@@ -748,7 +766,6 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
   a.k_chunk = kc;
   a.partial = nullptr;
   a.csplit = 1;
-  a.tiles_n = 0;
   if (splits > 1) {
     if (!ws || ws_bytes < simt_gemm_ws(p.M, p.N, splits))
       return fail(NK_ERR_WORKSPACE, "split-K needs %zu bytes of workspace",
@@ -779,21 +796,27 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
     if (p.sbn == 1) bmode = p.sbk % 4 == 0 && p.N % 4 == 0 && al16(p.B) ? L_MN16 : L_MN;
     else bmode = L_K;
     int bm = tile, bn = tile;
+    int sms = 0;
+    nk_status s = require_device(&sms);
+    if (s != NK_OK) return s;
     if (tile == 0) {
-      int sms = 0;
-      const nk_status s = require_device(&sms);
-      if (s != NK_OK) return s;
       const Choice c = choose(p.M, p.N, p.K, sms, splits == 1);
       bm = c.bm;
       bn = c.bn;
       a.csplit = c.csplit;
       if (a.csplit > 1) a.k_chunk = ((p.K + a.csplit - 1) / a.csplit + BK - 1) / BK * BK;
     }
-    a.tiles_n = (p.N + bn - 1) / bn;
-    const dim3 grid(a.tiles_n * a.csplit, (p.M + bm - 1) / bm, splits);
+    const dim3 grid((p.N + bn - 1) / bn * a.csplit, (p.M + bm - 1) / bm, splits);
     if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "M too large for the SIMT grid");
-    const nk_status s = bn == 128   ? launch_a<128, 128, 256>(a, amode, bmode, grid, st)
+    // A 64 x 64 tile that has an SM to itself and few steps: four warps of 8 x 4
+    // outputs cannot hide its start, eight of 4 x 4 do (us, 64 x 64 tiles:
+    // 128^3 7.3 / 6.0, 256^3 11.6 / 10.5, 8192 x 64 x 144 8.6 / 7.3; at K = 576 the
+    // larger blocks' fewer shared-memory reads win, 22.7 / 22.3 and, with A
+    // column-major, 19.8 / 21.8).
+    const bool alone = a.csplit == 1 && a.k_chunk <= 320 && (int64_t)grid.x * grid.y * grid.z <= sms;
+    s = bn == 128   ? launch_a<128, 128, 256>(a, amode, bmode, grid, st)
                         : bm == 128 ? launch_a<128, 64, 128>(a, amode, bmode, grid, st)
+                        : alone     ? launch_a<64, 64, 256>(a, amode, bmode, grid, st)
                                     : launch_a<64, 64, 128>(a, amode, bmode, grid, st);
     if (s != NK_OK || splits == 1) return s;
   }
