@@ -705,13 +705,16 @@ inline bool al16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) =
 // The built-in tile, and the CTAs that share a tile's reduction: the smallest
 // predicted time over the tiles and clusters of 1 to 8.  An SM works through
 // its units (tiles x slices) at the rate the tile's shape reaches, each unit
-// costs about a microsecond to fill and drain, and a cluster's exchange 1.6;
+// costs about a microsecond to fill and drain, and a cluster's exchange 1.9;
 // clusters of eight 128-row tiles pack badly.  The constants are fitted to
-// every combination timed on 27 shapes (products from 64^3 to 4096^3 and eight
-// convolutions), where the choice is 1.9 % off the best on average and 12 % at
-// worst.  Examples, us (tile / cluster): 256^3 64x64 / 1 12.3, / 8 5.3; 1024^3
-// 128x128 / 1 103, / 4 53; 1531 x 2047 x 1021 128x128 / 1 194, / 4 150;
-// 8x56x56x64 3x3 64x64 / 1 71, 128x64 / 2 52.
+// every combination timed on 34 products (64^3 to 2048^3, narrow and tall ones
+// among them, B in both layouts) and 14 convolutions, where the choice is 3.5 %
+// off the best of them on average and 22 % at worst.  (Clusters of 3, 5 and 6,
+// which the kernel does not form, would be ahead on some: 1531 x 2047 x 1021 in
+// clusters of 3, 142 us against 149.)  Examples, us (tile / cluster): 256^3
+// 64x64 / 1 12.3, / 8 5.3; 1024^3 128x128 / 1 103, / 4 53; 1531 x 2047 x 1021
+// 128x128 / 1 194, / 4 149; 8x56x56x64 3x3 64x64 / 1 71, 128x64 / 2 52; 700^3
+// 128x128 / 4 29.5, 64x64 / 4 23.5; 8192 x 64 x 576 128x64 / 4 26.1, 64x64 / 4 19.
 struct Choice {
   int bm, bn, csplit;
 };
@@ -720,7 +723,7 @@ Choice choose(int M, int N, int K, int sms, bool may_split) {
     int bm, bn, resident;
     double gflop_us;   // per SM
   };
-  static const Tile kTiles[] = {{128, 128, 2, 0.366}, {128, 64, 3, 0.352}, {64, 64, 2, 0.369}};
+  static const Tile kTiles[] = {{128, 128, 2, 0.357}, {128, 64, 3, 0.352}, {64, 64, 2, 0.368}};
   Choice best{128, 128, 1};
   double best_t = 1e30;
   for (const Tile& t : kTiles) {
@@ -731,12 +734,12 @@ Choice choose(int M, int N, int K, int sms, bool may_split) {
       // units of the busiest SM: whole ones while all are resident at once,
       // then the average and about half a set in the last wave
       const double u = units <= (int64_t)sms * t.resident ? (double)((units + sms - 1) / sms)
-                                                          : (double)units / sms + 0.51 * t.resident;
+                                                          : (double)units / sms + 0.515 * t.resident;
       const double warps = u * (t.bn == 128 ? 8 : 4);
-      const double fill = warps < 8 ? 0.624 : warps < 12 ? 0.864 : 1.0;   // too few to keep the FMA pipes busy
+      const double fill = warps < 8 ? 0.504 : warps < 12 ? 0.664 : 1.0;   // too few to keep the FMA pipes busy
       const double kc = ((K + cs - 1) / cs + BK - 1) / BK * BK;
-      const double pack = t.bm == 128 ? (cs == 8 ? 1.276 : cs == 4 ? 0.882 : 1.0) : 1.0;
-      const double us = u * (2e-6 * t.bm * t.bn * kc * pack / (t.gflop_us * fill) + 1.064) + (cs > 1 ? 1.642 : 0.0);
+      const double pack = t.bm == 128 ? (cs == 8 ? 1.214 : cs == 4 ? 0.882 : 1.0) : 1.0;
+      const double us = u * (2e-6 * t.bm * t.bn * kc * pack / (t.gflop_us * fill) + 1.026) + (cs > 1 ? 1.858 : 0.0);
       if (us < best_t) {
         best_t = us;
         best = {t.bm, t.bn, cs};
@@ -795,7 +798,7 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
     else amode = L_K;
     if (p.sbn == 1) bmode = p.sbk % 4 == 0 && p.N % 4 == 0 && al16(p.B) ? L_MN16 : L_MN;
     else bmode = L_K;
-    int bm = tile, bn = tile;
+    int bm = tile, bn = tile == 128 && p.N <= 64 ? 64 : tile;   // no empty half of a tile
     int sms = 0;
     nk_status s = require_device(&sms);
     if (s != NK_OK) return s;

@@ -55,6 +55,21 @@ def test_ragged_convolutions(nk, n, h, w, c, f, k, stride):
         assert np.array_equal(host(out), want)
 
 
+@pytest.mark.parametrize("M,N,K", [(700, 700, 700), (8192, 64, 576), (2500, 130, 400)])
+def test_built_in_tile_is_no_slower_than_plain_64(nk, M, N, K):
+    A, B, C = torch.ones(M, K, device=DEV), torch.ones(K, N, device=DEV), torch.empty(M, N, device=DEV)
+    t = []
+    for sched in (None, (64, 64, 16, 1, 2, 1)):
+        g = torch.cuda.CUDAGraph()
+        nk.nk_matmul(A, B, C, "f32", schedule=sched)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g):
+            for _ in range(8):
+                nk.nk_matmul(A, B, C, "f32", schedule=sched)
+        t.append(_time(g.replay))
+    assert t[0] <= 1.05 * t[1]
+
+
 def _time(call):
     for _ in range(3):
         call()
