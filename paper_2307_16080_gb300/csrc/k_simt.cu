@@ -21,6 +21,7 @@
 #include <atomic>
 #include <climits>
 #include <mutex>
+#include <type_traits>
 
 #include "nk_internal.cuh"
 
@@ -35,7 +36,8 @@ constexpr int THREADS = 256;
 // 4-byte copies, or in 16-byte ones where the operand's alignment allows them.
 // 16-byte copies along k store a tile of A as [m][k]; the others store [k][m]
 // and [k][n], 4-byte copies along k scattering a row of k.
-enum LoadMode { L_K = 0, L_MN = 1, L_MN16 = 2, L_CONV = 3, L_K16 = 4, L_CONV16 = 5 };
+// L_FAR and L_FAR16 are the gathers with 64-bit offsets and 32-bit positions.
+enum LoadMode { L_K = 0, L_MN = 1, L_MN16 = 2, L_CONV = 3, L_K16 = 4, L_CONV16 = 5, L_FAR = 6, L_FAR16 = 7 };
 
 struct KArgs {
   SimtGemm p;
@@ -133,8 +135,9 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
   constexpr int S = 4;                  // stages
   constexpr int RM = BM * BN / T >= 32 ? 8 : 4;   // rows of a thread
   constexpr int TY = BM / RM, TX = T / TY, TN = BN / TX;
-  constexpr bool CONV = AM == L_CONV || AM == L_CONV16;
-  constexpr bool AMK = AM == L_CONV16 || AM == L_K16;   // A is stored [m][k]
+  constexpr bool FAR = AM == L_FAR || AM == L_FAR16;
+  constexpr bool CONV = AM == L_CONV || AM == L_CONV16 || FAR;
+  constexpr bool AMK = AM == L_CONV16 || AM == L_K16 || AM == L_FAR16;   // A is stored [m][k]
   constexpr int A_LD = AMK ? BK + 4 : BM + 4, B_LD = BN + 4;
   constexpr int A_FL = AMK ? BM * A_LD : BK * A_LD;
   constexpr int STAGE = A_FL + BK * B_LD;
@@ -143,7 +146,10 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
   static_assert(TN == 8 || TN == 4, "8 x 8, 8 x 4 or 4 x 4 outputs per thread");
   static_assert(S * STAGE >= BM * BN, "a cluster's partial tiles reuse the ring");
   extern __shared__ __align__(16) float smem[];
-  __shared__ int row_off[BM], row_hw[BM];   // conv: offset of a row's first tap, and its (ih, iw)
+  // conv: offset of a row's first tap, and its (ih, iw), in one word unless they are far
+  using Off = typename std::conditional<FAR, int64_t, int>::type;
+  __shared__ Off row_off[BM];
+  __shared__ int row_hw[BM], row_w[FAR ? BM : 1];
   nk::pdl_wait();      // earlier kernels on the stream have finished
   nk::pdl_trigger();
   const SimtGemm& p = args.p;
@@ -164,15 +170,21 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
       const int m = min(m0 + r, p.M - 1);
       const int ow = m % g.ow, q = m / g.ow, oh = q % g.oh, n = q / g.oh;
       const int ih = oh * g.sh - g.pt, iw = ow * g.sw - g.pl;
-      row_off[r] = (int)(n * g.sin_n + ih * g.sin_h + iw * g.sin_w);
-      row_hw[r] = m0 + r < p.M ? (ih << 16) | (iw & 0xffff) : INT_MIN;   // past the end: above every input
+      row_off[r] = (Off)(n * g.sin_n + ih * g.sin_h + iw * g.sin_w);
+      // rows past the end: above every input
+      if constexpr (FAR) {
+        row_hw[r] = m0 + r < p.M ? ih : INT_MIN;
+        row_w[r] = iw;
+      } else {
+        row_hw[r] = m0 + r < p.M ? (ih << 16) | (iw & 0xffff) : INT_MIN;
+      }
     }
     __syncthreads();
   }
   // per-thread load positions, fixed for the whole loop
   const int lk = tid % BK, lr = tid / BK;          // along k: this thread's k and first row
   constexpr int LR = T / BK;
-  constexpr int KC = (AM == L_K16 || AM == L_CONV16) ? 4 : 1;   // k values a copy of A brings
+  constexpr int KC = AMK ? 4 : 1;   // k values a copy of A brings
   const int ak = tid % (BK / KC) * KC, ar = tid / (BK / KC);
   constexpr int AR = T * KC / BK;
   auto load_tile = [&](int t) {
@@ -191,12 +203,12 @@ __global__ void __launch_bounds__(T, T == 128 ? 3 : 2) simt_gemm_kernel(const __
       const int tap = kc / g.c, c = kc - tap * g.c;
       const int kh = tap / g.kw, kw = tap - kh * g.kw;
       const int dh = kh * g.dh, dw = kw * g.dw;
-      const int d = (int)(dh * g.sin_h + dw * g.sin_w) + c;
+      const Off d = (Off)(dh * g.sin_h + dw * g.sin_w) + c;
 #pragma unroll
       for (int i = 0; i < BM / AR; ++i) {
         const int r = ar + i * AR;
         const int hw = row_hw[r];
-        const int ih = (hw >> 16) + dh, iw = (int)(short)(hw & 0xffff) + dw;
+        const int ih = (FAR ? hw : hw >> 16) + dh, iw = (FAR ? row_w[r] : (int)(short)(hw & 0xffff)) + dw;
         const bool in = ok && (unsigned)ih < (unsigned)g.h && (unsigned)iw < (unsigned)g.w;
         cpa(sa + (uint32_t)((AMK ? r * A_LD + ak : ak * A_LD + r) * 4), p.A + (in ? row_off[r] + d : 0), in);
       }
@@ -648,9 +660,9 @@ __global__ void __launch_bounds__(256) splitk_reduce4_kernel(const __grid_consta
 template <int BM, int BN, int T, int AM, int BMD>
 nk_status launch_kernel(const KArgs& a, dim3 grid, cudaStream_t st) {
   auto kern = simt_gemm_kernel<BM, BN, T, AM, BMD>;
-  constexpr bool amk = AM == L_K16 || AM == L_CONV16;
+  constexpr bool amk = AM == L_K16 || AM == L_CONV16 || AM == L_FAR16;
   constexpr int smem = 4 * ((amk ? BM * (BK + 4) : BK * (BM + 4)) + BK * (BN + 4)) * (int)sizeof(float);
-  if constexpr (smem + 2 * BM * (int)sizeof(int) > 48 * 1024) {
+  if constexpr (smem + 16 * BM > 48 * 1024) {
     static std::atomic<bool> set[64];   // per device; setting it twice is harmless
     int dev = 0;
     cudaGetDevice(&dev);
@@ -686,6 +698,16 @@ nk_status launch_a(const KArgs& a, int amode, int bmode, dim3 grid, cudaStream_t
     case L_CONV16:
       return bmode == L_MN16 ? launch_kernel<BM, BN, T, L_CONV16, L_MN16>(a, grid, st)
                              : launch_kernel<BM, BN, T, L_CONV16, L_MN>(a, grid, st);
+    case L_FAR16:   // (one tile width is enough)
+      if constexpr (BN == 64 && T == 128)
+        return bmode == L_MN16 ? launch_kernel<BM, BN, T, L_FAR16, L_MN16>(a, grid, st)
+                               : launch_kernel<BM, BN, T, L_FAR16, L_MN>(a, grid, st);
+      return fail(NK_ERR_UNSUPPORTED, "no such FP32 tile");
+    case L_FAR:
+      if constexpr (BN == 64 && T == 128)
+        return bmode == L_MN16 ? launch_kernel<BM, BN, T, L_FAR, L_MN16>(a, grid, st)
+                               : launch_kernel<BM, BN, T, L_FAR, L_MN>(a, grid, st);
+      return fail(NK_ERR_UNSUPPORTED, "no such FP32 tile");
     default:   // a convolution's filters are row-major [K][F]
       return bmode == L_MN16 ? launch_kernel<BM, BN, T, L_CONV, L_MN16>(a, grid, st)
                              : launch_kernel<BM, BN, T, L_CONV, L_MN>(a, grid, st);
@@ -775,14 +797,17 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
                   simt_gemm_ws(p.M, p.N, splits));
     a.partial = static_cast<float*>(ws);
   }
-  // The gather keeps a pixel's offset in 32 bits and its position in 16.
+  // The gather keeps a pixel's offset in 32 bits and its position in 16; long
+  // signals and inputs beyond 2^30 values take the one with 64 and 32 (1 x 1 x
+  // 40000 x 64 -> 64, 1 x 3: 139 us with the register-loading kernel, which
+  // runs programs, 29 with this one).
   const ConvGeom& cg = p.conv;
   const bool far = p.is_conv && (cg.h + cg.pt + cg.kh * cg.dh > 32000 || cg.w + cg.pl + cg.kw * cg.dw > 32000 ||
                                  cg.oh * (int64_t)cg.sh > 32000 || cg.ow * (int64_t)cg.sw > 32000 ||
                                  cg.n * cg.sin_n + (cg.h + cg.pt + cg.kh * cg.dh) * cg.sin_h +
                                          (cg.w + cg.pl + cg.kw * cg.dw) * cg.sin_w >=
                                      INT32_MAX / 2);
-  if (p.pro_a.n || p.pro_b.n || p.ew.n || far) {
+  if (p.pro_a.n || p.pro_b.n || p.ew.n) {
     if (tile == 0) tile = (int64_t)((p.M + 127) / 128) * ((p.N + 127) / 128) < 152 ? 64 : 128;
     const dim3 grid((p.N + tile - 1) / tile, (p.M + tile - 1) / tile, splits);
     if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "M too large for the SIMT grid");
@@ -792,7 +817,8 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
     // Pick the load modes from the layout and alignment.
     int amode, bmode;
     if (p.is_conv)
-      amode = cg.c % 4 == 0 && cg.sin_n % 4 == 0 && cg.sin_h % 4 == 0 && cg.sin_w % 4 == 0 && al16(p.A) ? L_CONV16 : L_CONV;
+      amode = cg.c % 4 == 0 && cg.sin_n % 4 == 0 && cg.sin_h % 4 == 0 && cg.sin_w % 4 == 0 && al16(p.A) ? (far ? L_FAR16 : L_CONV16)
+                                                                                                           : (far ? L_FAR : L_CONV);
     else if (p.sak == 1 && p.sam % 4 == 0 && p.K % 4 == 0 && al16(p.A)) amode = L_K16;
     else if (p.sam == 1 && p.sak != 1) amode = p.sak % 4 == 0 && p.M % 4 == 0 && al16(p.A) ? L_MN16 : L_MN;
     else amode = L_K;
@@ -809,6 +835,7 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
       a.csplit = c.csplit;
       if (a.csplit > 1) a.k_chunk = ((p.K + a.csplit - 1) / a.csplit + BK - 1) / BK * BK;
     }
+    if (far) bn = 64;
     const dim3 grid((p.N + bn - 1) / bn * a.csplit, (p.M + bm - 1) / bm, splits);
     if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "M too large for the SIMT grid");
     // A 64 x 64 tile that has an SM to itself and few steps: four warps of 8 x 4
@@ -816,7 +843,7 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
     // 128^3 7.3 / 6.0, 256^3 11.6 / 10.5, 8192 x 64 x 144 8.6 / 7.3; at K = 576 the
     // larger blocks' fewer shared-memory reads win, 22.7 / 22.3 and, with A
     // column-major, 19.8 / 21.8).
-    const bool alone = a.csplit == 1 && a.k_chunk <= 320 && (int64_t)grid.x * grid.y * grid.z <= sms;
+    const bool alone = !far && a.csplit == 1 && a.k_chunk <= 320 && (int64_t)grid.x * grid.y * grid.z <= sms;
     s = bn == 128   ? launch_a<128, 128, 256>(a, amode, bmode, grid, st)
                         : bm == 128 ? launch_a<128, 64, 128>(a, amode, bmode, grid, st)
                         : alone     ? launch_a<64, 64, 256>(a, amode, bmode, grid, st)
