@@ -800,7 +800,7 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
   // The gather keeps a pixel's offset in 32 bits and its position in 16; long
   // signals and inputs beyond 2^30 values take the one with 64 and 32 (1 x 1 x
   // 40000 x 64 -> 64, 1 x 3: 139 us with the register-loading kernel, which
-  // runs programs, 29 with this one).
+  // runs programs, 32 with this one).
   const ConvGeom& cg = p.conv;
   const bool far = p.is_conv && (cg.h + cg.pt + cg.kh * cg.dh > 32000 || cg.w + cg.pl + cg.kw * cg.dw > 32000 ||
                                  cg.oh * (int64_t)cg.sh > 32000 || cg.ow * (int64_t)cg.sw > 32000 ||
@@ -808,7 +808,9 @@ nk_status simt_gemm(const SimtGemm& p, int tile, int splits, void* ws, size_t ws
                                          (cg.w + cg.pl + cg.kw * cg.dw) * cg.sin_w >=
                                      INT32_MAX / 2);
   if (p.pro_a.n || p.pro_b.n || p.ew.n) {
-    if (tile == 0) tile = (int64_t)((p.M + 127) / 128) * ((p.N + 127) / 128) < 152 ? 64 : 128;
+    // Convolutions have few columns: a 128-wide tile is half empty at 64 filters
+    // (8x56x56x64 3x3 + GELU 174 us with 64 x 64 tiles, 260 with 128 x 128).
+    if (tile == 0) tile = p.is_conv || (int64_t)((p.M + 127) / 128) * ((p.N + 127) / 128) < 152 ? 64 : 128;
     const dim3 grid((p.N + tile - 1) / tile, (p.M + tile - 1) / tile, splits);
     if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "M too large for the SIMT grid");
     const nk_status s = tile == 128 ? launch_fused<2, 2>(a, grid, st) : launch_fused<1, 1>(a, grid, st);
