@@ -15,6 +15,7 @@
 #include <cuda_fp8.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 
 #include "nk_internal.cuh"
@@ -175,6 +176,38 @@ struct Caster<2> {
   }
 };
 
+// Row-major cast whose output rows take no word stores: neighbouring lanes take
+// neighbouring elements, eight each, 2^tx_log apart.
+template <int KIND, bool PRO>
+__global__ void __launch_bounds__(256) cast_rows_single(const float* in, int64_t rows, int64_t cols, int64_t ld_in,
+                                                        const float* amax, typename Caster<KIND>::T* __restrict__ o0,
+                                                        typename Caster<KIND>::T* __restrict__ o1, int64_t ld_out,
+                                                        float* scale_out, int tx_log, const __grid_constant__ EwProg pro) {
+  nk::pdl_wait();      // earlier kernels on the stream have finished
+  nk::pdl_trigger();
+  using T = typename Caster<KIND>::T;
+  constexpr int V = 8;
+  const float s = KIND == 1 ? fp8_scale_of(amax) : 1.f;
+  if (scale_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *scale_out = s;
+  const int ty = 256 >> tx_log;
+  const int64_t c = ((int64_t)blockIdx.x << tx_log) * V + (threadIdx.x & ((1 << tx_log) - 1));
+  for (int64_t r = (int64_t)blockIdx.y * ty + (threadIdx.x >> tx_log); r < rows; r += (int64_t)gridDim.y * ty) {
+    float v[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) v[j] = c + (j << tx_log) < cols ? in[r * ld_in + c + (j << tx_log)] : 0.f;
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      const int64_t cc = c + (j << tx_log);
+      if (cc >= cols) break;
+      if constexpr (PRO) v[j] = ew_run(pro, v[j], r * ld_in + cc);
+      T a, b;
+      Caster<KIND>::cvt(v[j], s, a, b);
+      o0[r * ld_out + cc] = a;
+      if (KIND == 2) o1[r * ld_out + cc] = b;
+    }
+  }
+}
+
 // Row-major cast without transpose: eight elements per thread per step, read
 // as two 16-byte words (one by one where the input's alignment does not allow
 // it) and written as one 16-byte word of BF16 (8 bytes of E4M3).  HBM-bound; a
@@ -194,14 +227,12 @@ __global__ void __launch_bounds__(256) cast_rows(const float* in, int64_t rows, 
   constexpr int V = 8;
   const float s = KIND == 1 ? fp8_scale_of(amax) : 1.f;
   if (scale_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *scale_out = s;
+  constexpr int OB = V * (int)sizeof(T);   // bytes of an output word: 16 (BF16) or 8 (E4M3)
   const int64_t c = (((int64_t)blockIdx.x << tx_log) + (threadIdx.x & ((1 << tx_log) - 1))) * V;
-  if (c >= cols) return;
   const int ty = 256 >> tx_log;
+  if (c >= cols) return;
   const bool whole = c + V <= cols;
   const bool vin = whole && (ld_in % 4 == 0) && ((reinterpret_cast<uintptr_t>(in) & 15) == 0);
-  constexpr int OB = V * (int)sizeof(T);   // bytes of an output word: 16 (BF16) or 8 (E4M3)
-  const bool vout = whole && (ld_out * (int64_t)sizeof(T)) % OB == 0 && (reinterpret_cast<uintptr_t>(o0) & (OB - 1)) == 0 &&
-                    (KIND != 2 || (reinterpret_cast<uintptr_t>(o1) & (OB - 1)) == 0);
   for (int64_t r = (int64_t)blockIdx.y * ty + (threadIdx.x >> tx_log); r < rows; r += (int64_t)gridDim.y * ty) {
     const float* src = in + r * ld_in + c;
     float v[V];
@@ -223,7 +254,7 @@ __global__ void __launch_bounds__(256) cast_rows(const float* in, int64_t rows, 
 #pragma unroll
     for (int j = 0; j < V; ++j) Caster<KIND>::cvt(v[j], s, a[j], b[j]);
     T* d0 = o0 + r * ld_out + c;
-    if (vout) {
+    if (whole) {
       if constexpr (OB == 16) {
         *reinterpret_cast<uint4*>(d0) = *reinterpret_cast<const uint4*>(a);
         if (KIND == 2) *reinterpret_cast<uint4*>(o1 + r * ld_out + c) = *reinterpret_cast<const uint4*>(b);
@@ -240,6 +271,37 @@ __global__ void __launch_bounds__(256) cast_rows(const float* in, int64_t rows, 
       }
     }
   }
+}
+
+// Transposing cast of a matrix with few rows or few columns, most of whose
+// tile below would be empty: a thread takes one position of the long side and
+// walks the short one.  us, with the tile / this: 3 x 1000000 to E4M3 57 / 9,
+// 1000000 x 3 33 / 13.
+template <int KIND, bool PRO>
+__global__ void __launch_bounds__(256) cast_transpose_few(const float* in, int64_t rows, int64_t cols, int64_t ld_in,
+                                                          const float* amax,
+                                                          typename Caster<KIND>::T* __restrict__ o0,
+                                                          typename Caster<KIND>::T* __restrict__ o1, int64_t ld_out,
+                                                          float* scale_out, bool few_rows,
+                                                          const __grid_constant__ EwProg pro) {
+  nk::pdl_wait();      // earlier kernels on the stream have finished
+  nk::pdl_trigger();
+  using T = typename Caster<KIND>::T;
+  const float s = KIND == 1 ? fp8_scale_of(amax) : 1.f;
+  if (scale_out && blockIdx.x == 0 && threadIdx.x == 0) *scale_out = s;
+  const int64_t n = few_rows ? cols : rows;
+  const int m = (int)(few_rows ? rows : cols);
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
+#pragma unroll 4
+    for (int k = 0; k < m; ++k) {
+      const int64_t r = few_rows ? k : i, c = few_rows ? i : k;
+      float v = in[r * ld_in + c];
+      if constexpr (PRO) v = ew_run(pro, v, r * ld_in + c);
+      T a, b;
+      Caster<KIND>::cvt(v, s, a, b);
+      o0[c * ld_out + r] = a;
+      if (KIND == 2) o1[c * ld_out + r] = b;
+    }
 }
 
 // Transposing cast: a tile of 64 input columns by 32 words of P rows through
@@ -408,8 +470,22 @@ nk_status launch_cast(const float* in, int64_t rows, int64_t cols, int64_t ld_in
     constexpr int TR = 32 * (4 / (int)sizeof(T));   // rows of a tile (cast_transpose)
     dim3 grid((unsigned)((cols + 63) / 64), (unsigned)((rows + TR - 1) / TR));
     if (grid.y > 65535) return fail(NK_ERR_UNSUPPORTED, "too many rows for the transposing cast");
+    const bool few_rows = rows * 4 <= TR && rows <= cols;   // a quarter of a tile
+    if (few_rows || cols <= 16) {
+      const int64_t blocks = ((few_rows ? cols : rows) + 255) / 256;
+      (void)nk::launch_k(cast_transpose_few<KIND, PRO>, dim3((unsigned)std::min<int64_t>(blocks, (int64_t)sms * 64)), dim3(256),
+                         0, st, 1, in, rows, cols, ld_in, amax, o0, o1, ld_out, scale_out, few_rows, pro);
+      return check_launch("cast kernel");
+    }
     (void)nk::launch_k(cast_transpose<KIND, PRO>, dim3(grid), dim3(256), 0, st, 1, in, rows, cols, ld_in, amax, o0, o1, ld_out, scale_out, pro);
   } else {
+    // a dense matrix whose rows do not end on words is one long row of them
+    // (us: 1001 x 1003 to BF16 3.6 / 1.9, 1000000 x 3 6.4 / 4.4)
+    if (ld_in == cols && ld_out == cols && cols % 8 != 0) {
+      cols *= rows;
+      ld_in = ld_out = cols + (8 - cols % 8) % 8;   // one row: only the alignment of the strides is looked at
+      rows = 1;
+    }
     const int64_t chunks = (cols + 7) / 8;
     int tx_log = 0;
     while (tx_log < 8 && (int64_t(1) << tx_log) < chunks) ++tx_log;
@@ -420,8 +496,11 @@ nk_status launch_cast(const float* in, int64_t rows, int64_t cols, int64_t ld_in
     const int64_t cap = ((int64_t)sms * 32 + bx - 1) / bx;   // a few waves of eight resident blocks
     if (by > cap) by = cap;
     if (by > 65535) by = 65535;
-    (void)nk::launch_k(cast_rows<KIND, PRO>, dim3((unsigned)bx, (unsigned)by), dim3(256), 0, st, 1, in, rows, cols, ld_in,
-                       amax, o0, o1, ld_out, scale_out, tx_log, pro);
+    constexpr uintptr_t OB = 8 * sizeof(T);   // an output word: eight values
+    const bool words = ld_out * sizeof(T) % OB == 0 && reinterpret_cast<uintptr_t>(o0) % OB == 0 &&
+                       (KIND != 2 || reinterpret_cast<uintptr_t>(o1) % OB == 0);
+    (void)nk::launch_k(words ? cast_rows<KIND, PRO> : cast_rows_single<KIND, PRO>, dim3((unsigned)bx, (unsigned)by),
+                       dim3(256), 0, st, 1, in, rows, cols, ld_in, amax, o0, o1, ld_out, scale_out, tx_log, pro);
   }
   return check_launch("cast kernel");
 }
