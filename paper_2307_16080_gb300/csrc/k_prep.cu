@@ -79,7 +79,14 @@ __global__ void __launch_bounds__(256, PRO ? 2 : 5) amax_stage1(const float* x, 
 #pragma unroll
       for (int u = 0; u < 8; ++u) fold(v[u], i + u * stride);
     }
-    for (; i < n4; i += stride) fold(x4[i], i);
+    // and in the last, partial round (3 M values: 3.8 us, 4.8 one by one)
+    float4 v[7];
+#pragma unroll
+    for (int u = 0; u < 7; ++u)
+      if (i + u * stride < n4) v[u] = x4[i + u * stride];
+#pragma unroll
+    for (int u = 0; u < 7; ++u)
+      if (i + u * stride < n4) fold(v[u], i + u * stride);
   } else {
     // strided rows: blocks stride over rows, threads over the row
     const bool vec = al && (cols % 4 == 0) && (ld % 4 == 0);
@@ -574,13 +581,19 @@ nk_status prep_amax(const float* x, int64_t rows, int64_t cols, int64_t ld, floa
   if (!x) return fail(NK_ERR_INVALID_ARG, "amax: null pointer");
   if (!ws || ws_bytes < prep_amax_ws(rows * cols))
     return fail(NK_ERR_WORKSPACE, "amax needs %zu bytes of workspace", prep_amax_ws(rows * cols));
-  if (pro && pro->n)
-    (void)nk::launch_k(amax_stage1<true>, dim3(kAmaxBlocks), dim3(256), 0, st, 1, x, rows, cols, ld, static_cast<float*>(ws), *pro);
-  else
-    (void)nk::launch_k(amax_stage1<false>, dim3(kAmaxBlocks), dim3(256), 0, st, 1, x, rows, cols, ld, static_cast<float*>(ws), EwProg{});
-  nk_status s = check_launch("amax_stage1");
+  // one wave of the five blocks an SM holds, fewer for a short dense run (at
+  // most four words a thread; 500 thousand values: 2.8 us, 3.4 with 1024 blocks)
+  int sms = 0;
+  nk_status s = require_device(&sms);
   if (s != NK_OK) return s;
-  (void)nk::launch_k(amax_stage2, dim3(1), dim3(1024), 0, st, 1, static_cast<float*>(ws), kAmaxBlocks, amax);
+  int blocks = std::min(kAmaxBlocks, 5 * sms);
+  if (ld == cols) blocks = (int)std::min<int64_t>(blocks, (rows * cols + 4095) / 4096);
+  if (pro && pro->n)
+    (void)nk::launch_k(amax_stage1<true>, dim3(blocks), dim3(256), 0, st, 1, x, rows, cols, ld, static_cast<float*>(ws), *pro);
+  else
+    (void)nk::launch_k(amax_stage1<false>, dim3(blocks), dim3(256), 0, st, 1, x, rows, cols, ld, static_cast<float*>(ws), EwProg{});
+  if ((s = check_launch("amax_stage1")) != NK_OK) return s;
+  (void)nk::launch_k(amax_stage2, dim3(1), dim3(1024), 0, st, 1, static_cast<float*>(ws), blocks, amax);
   return check_launch("amax_stage2");
 }
 

@@ -1,5 +1,6 @@
 """Conversions of narrow and of few-row matrices, of dense matrices whose rows
-do not end on words: bit for bit, and cheaper than a whole tile of the transpose
+do not end on words, and amax of short runs: bit for bit, with NaN and the last
+element in every position class, and no slower than the kernels for whole tiles
 (3 x 1000000 took nearly as long as 24 rows)."""
 import pytest
 import torch
@@ -35,6 +36,16 @@ def test_narrow_casts_bitwise(rows, cols, pad_in, pad_out, transpose):
     assert torch.equal(q.t, (want * 128).to(torch.float8_e4m3fn).contiguous().view(torch.uint8))
     for o in outs + [q]:
         o.check()
+
+
+@pytest.mark.parametrize("n", [4, 1020, 1024, 1028, 4096, 1024 * 1024, 7 * 1024 * 1024 + 4])
+def test_amax_of_short_runs(n):
+    x, out = torch.zeros(n, device=DEV), torch.empty(1, device=DEV)
+    for i, at in enumerate((0, n // 2, n - 1)):
+        x[at] = -5.0 - i
+        assert host(nk.nk_amax(x, out))[0] == 5.0 + i
+    x[n - 2] = float("nan")
+    assert torch.isnan(nk.nk_amax(x, out)).item()
 
 
 def _time(run):
