@@ -304,7 +304,10 @@ def _conv_args(stride, dilation, pad):
 
 
 def _conv_bytes(stride, dilation, pad):
-    return _PAIR.pack(*stride), _PAIR.pack(*dilation), _QUAD.pack(*pad)
+    try:
+        return _PAIR.pack(*stride), _PAIR.pack(*dilation), _QUAD.pack(*pad)
+    except struct.error:   # fewer numbers, which the arrays fill up with zeros, or ones that they refuse
+        return _conv_args(stride, dilation, pad)
 
 
 def nk_conv2d_workspace_size(I, W, O, stride=(1, 1), dilation=(1, 1), pad=(0, 0, 0, 0),
