@@ -298,10 +298,7 @@ nk_status plan_matmul(const nk_tensor* A, const nk_tensor* B, const nk_tensor* C
     P.total = align_up(P.kern_bytes);
     return NK_OK;
   }
-  // Rows of the converted operands: whole 128-byte lines once they are several
-  // lines long, because a TMA row of 128 bytes that straddles two lines costs
-  // the L2 two; short rows stay packed.
-  P.ldk = P.K >= 256 ? round_up(P.K, 128 / esz) : round_up(P.K, 16);
+  P.ldk = tc_operand_ld(kind, P.K);
   size_t off = 0;
   const size_t a_bytes = align_up((size_t)P.M * P.ldk * esz);
   const size_t b_bytes = align_up((size_t)P.N * P.ldk * esz);

@@ -203,6 +203,15 @@ namespace nk {
 // (A2/B2 hold the lo halves).  alpha = 1/(sa*sb) when scale pointers are set.
 enum TcKind { TC_BF16 = 0, TC_FP8 = 1, TC_BF16X3 = 2 };
 
+// Row stride (elements) of converted operands: whole 128-byte lines once rows
+// are several lines long, because a TMA row of 128 bytes that straddles two
+// lines costs the L2 two; short rows stay packed.  The calls and the tuner's
+// timings lay their operands out alike.
+inline int64_t tc_operand_ld(int kind, int64_t K) {
+  const int64_t unit = K < 256 ? 16 : kind == TC_FP8 ? 128 : 64;
+  return (K + unit - 1) / unit * unit;
+}
+
 struct TcGemm {
   int kind;
   int M, N, K;

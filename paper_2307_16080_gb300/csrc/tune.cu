@@ -209,7 +209,7 @@ struct Runner {
     if (p->op == NK_OP_MATMUL) {
       const int kind = kind_of(p->precision);
       const int esz = kind == TC_FP8 ? 1 : 2;
-      const int64_t ld = (K + 15) / 16 * 16;
+      const int64_t ld = tc_operand_ld(kind, K);
       const size_t a = (size_t)M * ld * esz, b = (size_t)N * ld * esz;
       const size_t parts = kind == TC_BF16X3 ? 2 : 1;
       op_bytes = parts * (a + b);
