@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(128, rows_ctas(KH, CO)) direct_rows_kernel(con
   const int n = blockIdx.y / groups;
   const int co0 = (blockIdx.y % groups) * CO;
   const int ncog = min(CO, p.CO - co0);
-  if (wo - lane * 4 >= p.OW) return;   // whole warps: the stores shuffle
+  if (wo - lane * 4 >= p.OW) return;   // whole warps: the votes below ask every lane
   float acc[ROWS][CO][4];
 #pragma unroll
   for (int r = 0; r < ROWS; ++r)
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(128) direct_stream_kernel(const __grid_constan
   const int n = blockIdx.z / groups;
   const int co0 = (blockIdx.z % groups) * CO;
   const int ncog = min(CO, p.CO - co0);
-  if (wo - lane * 4 >= p.OW || ho0 >= p.OH) return;   // whole warps: the stores shuffle
+  if (wo - lane * 4 >= p.OW || ho0 >= p.OH) return;   // whole warps: the votes below ask every lane
   const int rows = min(rpt, p.OH - ho0);
   float w[CO][TAPS];
 #pragma unroll
@@ -455,6 +455,8 @@ nk_status launch_registers(const Direct& p, cudaStream_t st) {
   if (s != NK_OK) return s;
   const int groups = (p.CO + 3) / 4;
   if ((int64_t)p.N * groups > 65535) return fail(NK_ERR_UNSUPPORTED, "batch x channel groups too large");
+  // the limit of a grid of row blocks, which the kernels for one input channel
+  // (64 rows a block at most) and for several (4) are held to
   if ((p.OH - 1) / (p.CI == 1 ? 64 : 4) >= 65535) return fail(NK_ERR_UNSUPPORTED, "output too tall");
   if constexpr (KH < 5) {
     if (p.CI == 1 && (KH == 3 || p.CO == 1)) {

@@ -968,8 +968,9 @@ extern "C" nk_status nk_matmul_f32_splitk_noalloc(const float* A, int64_t lda, c
   p.C = C; p.scm = ldc; p.scn = 1;
   p.M = M; p.N = N; p.K = K;
   p.alpha = 1.f; p.beta = 0.f;
-  // The tile nk_matmul's FP32 rule picks: 64 x 64 while 128 x 128 tiles
-  // would not give every SM one.
+  // 64 x 64 tiles while 128 x 128 ones would not give every SM one (the caller
+  // has chosen the slices, so the built-in rule, which slices K itself, has no
+  // say).
   const int tile = (int64_t)((M + 127) / 128) * ((N + 127) / 128) < sms ? 64 : 128;
   // Every slice overwrites its whole [M,N] partial tile, so the scratch needs
   // no clearing between calls.

@@ -73,7 +73,8 @@ bool is_wide(int kind, const nk_schedule& s) { return s.tile_n == 512 || (kind =
 // fitted: 0.62 per 64-deep K block + 1.5 (128 x 128), 1.0 + 6 (wide).  Whole
 // calls, 128 x 128 against wide: 4096^3 329 / 311 us, 4096 x 4096 x 1024 92 /
 // 96, 1024 x 4096 x 1024 33.0 / 32.2, 3001 x 2002 x 1999 87 / 99.  The schedule
-// space has no such point: a caller's schedule is always taken as it is.
+// space, whose points the stored corpora time one by one, does not hold this one:
+// it cannot be asked for, and a caller's schedule is always taken as it is.
 bool x3_wide_wins(int M, int N, int K, int sms) {
   const int64_t wide = (int64_t)((M + 255) / 256) * ((N + 255) / 256);
   const int64_t square = (int64_t)((M + 127) / 128) * ((N + 127) / 128);
@@ -414,12 +415,12 @@ nk_schedule tc_conv_default_schedule(const ConvGeom& g, int F, int sms, int kind
   const int tiles = ctiles * ((F + s.tile_n - 1) / s.tile_n);
   const int nkb = g.kh * g.kw * t.cblocks;
   // More than a wave of two CTAs per SM, and enough K blocks to cover a tile's
-  // epilogue (with fewer than 16, a wave and a half): 256 x 128 tiles on CTA pairs (three stages, so that two CTAs
-  // still share an SM), which read the filters half as often.  128 x 64 tiles /
-  // pairs, us: 128x56x56x64 -> 128 3x3 / 2 32.4 / 22.4, 64x28x28x128 -> 256 3x3 /
-  // 2 21.3 / 15.6, 128x14x14x256 -> 512 3x3 / 2 37.1 / 23.5; with one wave,
-  // 32x28x28x128 -> 256 3x3 / 2 13.0 / 14.0; with four K blocks, 128x14x14x256
-  // -> 512 1x1 / 2 8.5 / 9.0.
+  // epilogue (with fewer than 16, a wave and a half): 256 x 128 tiles on CTA
+  // pairs (three stages, so that two CTAs still share an SM), which read the
+  // filters half as often.  128 x 64 tiles / pairs, us: 128x56x56x64 -> 128 3x3 /
+  // 2 32.4 / 22.4, 64x28x28x128 -> 256 3x3 / 2 21.3 / 15.6, 128x14x14x256 -> 512
+  // 3x3 / 2 37.1 / 23.5; with one wave, 32x28x28x128 -> 256 3x3 / 2 13.0 / 14.0;
+  // with four K blocks, 128x14x14x256 -> 512 1x1 / 2 8.5 / 9.0.
   if (kind == TC_BF16 && F > 64 && ((tiles > 2 * sms && nkb >= 16) || (tiles > 3 * sms && nkb >= 8)))
     return nk_schedule{256, 128, 64, 2, 3, 1};
   while (tiles * s.split_k * 2 <= sms && nkb / (s.split_k * 2) >= 4 && s.split_k < 16) s.split_k *= 2;

@@ -877,9 +877,14 @@ nk_schedule tc_halo_default_schedule(const ConvGeom& g, int F, int sms, bool* ok
     const nk_schedule d{256, 64, cb * g.kh, 1, 2, 1};
     if (units >= 4 * (int64_t)sms && halo_schedule_valid(g, F, d, kind)) {
       // With more than one channel block and more than one filter tile that
-      // many units are faster on CTA pairs, per tap (tc_conv_default_schedule):
+      // many units are faster per tap (tc_conv_default_schedule): on CTA pairs
       // 128x28x28x128 50.3 / 33.3 us, 128x14x14x256 55.3 / 39.3, 32x40x40x160
-      // 59.4 / 44.4, 128x33x33x72 193 / 79.
+      // 59.4 / 44.4, 128x33x33x72 193 / 79.  Small images have several times
+      // more windows than per-tap tiles, and where those are too few for pairs
+      // the rule there takes 128 x 64 tiles, which are the fastest of all four:
+      // this kernel with two buffers / one / pairs / 128 x 64, 512x4x4x128 -> 256
+      // 21.9 / 18.0 / 13.7 / 13.1 us, 512x3x3x256 -> 256 38.8 / 28.2 / 21.0 / 19.4,
+      // 90x10x10x128 -> 256 22.1 / 18.0 / 13.4 / 12.6.
       if (kind == TC_BF16 && g.c > 64 && F > 64) return best;
       s = d;
     }

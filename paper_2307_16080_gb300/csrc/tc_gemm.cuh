@@ -20,8 +20,9 @@
 //               next tile's main loop through the second accumulator.
 //
 // BF16x3 sums hi*hi, hi*lo and lo*hi per K step: on one CTA in two MMAs, hi *
-// [hi lo] over two adjacent accumulators and lo * hi into the second.  Split-K writes each slice's raw tile to the workspace and the
-// fixed-order warp-shuffle reduce applies the epilogue.
+// [hi lo] over two adjacent accumulators and lo * hi into the second.  Split-K
+// writes each slice's raw tile to the workspace and a fixed-order reduce pass
+// applies the epilogue.
 //
 // Every wait is bounded (see tc_ptx.cuh); on a timeout the CTA drains its own
 // copies and MMAs, frees TMEM and exits, and the host reports NK_ERR_TIMEOUT.
