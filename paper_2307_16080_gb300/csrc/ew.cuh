@@ -42,11 +42,11 @@ inline EwProg ew_shift(EwProg e, int64_t off) {
 // elements in flight: GELU with erfcf 141 cycles, x / (1 + e) with the
 // division 105, tanhf 28, expf 17).
 
-// n / d for d in [2^-64, 2^64]: the hardware reciprocal and one residual
-// correction of the quotient (Markstein, "Computation of elementary functions
-// on the IBM RISC System/6000", 1990), which leaves the rounding of an exact
-// division (to 2^-44).  Where an infinite n makes the residual a NaN, and for a
-// zero n, whose sign it would lose, the uncorrected quotient stands.
+// n / d for d in [1, 2^93]: the hardware reciprocal and one residual correction
+// of the quotient (Markstein, "Computation of elementary functions on the IBM
+// RISC System/6000", 1990), which leaves the rounding of an exact division (to
+// 2^-44).  Where an infinite n makes the residual a NaN, and for a zero n, whose
+// sign it would lose, the uncorrected quotient stands.
 static __device__ __forceinline__ float ew_div(float n, float d) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
@@ -57,14 +57,13 @@ static __device__ __forceinline__ float ew_div(float n, float d) {
 // y * sigmoid(u) = y / (1 + e^-u): three roundings, as with an IEEE division.
 // (y e^u / (1 + e^u) for every u < 0 has a fourth: the worst relative error of
 // SiLU was 2.5e-7 that way, on 600 thousand values, and is under 2.4e-7.)
-// Below -64, where 1 + e^-u is e^-u, both sides are scaled by 2^-64 so that the
-// reciprocal stays a normal number; below -88, where e^-u nears the end of
-// FP32, y e^u keeps the results that a division by infinity loses.
+// Below -64 1 + e^-u is e^-u in FP32, and y e^u is the quotient with two; it
+// also keeps the results below -88.7 that a division by infinity loses (the
+// 1.4 above that, where e^u is subnormal, to 5e-7).
 static __device__ __forceinline__ float ew_logistic(float y, float u) {
-  const bool low = u < -64.f, deep = u < -88.f;
-  const float e = expf(deep ? u : -u);
-  const float s = low ? 0x1p-64f : 1.f;
-  return ew_div(y * (deep ? e : s), deep ? 1.f : fmaf(e, s, low ? 0.f : 1.f));
+  const bool low = u < -64.f;
+  const float e = expf(low ? u : -u);
+  return ew_div(low ? y * e : y, low ? 1.f : 1.f + e);
 }
 
 // x * Phi(x).  With a = |x|, Phi(-a) = exp(-a^2 / 2) R(a), where R is half the

@@ -574,7 +574,10 @@ __global__ void __launch_bounds__((WIDE || EP8) ? 320 : 192, (WIDE || EP8 || KIN
           const uint32_t ta0 = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * acc_cols + c_begin);
           const float bm = (t.bias && p.bias_on_m && row_ok) ? t.bias[row] : 0.f;
           constexpr int PARTS = KIND == TC_BF16X3 ? 2 : 1;
-          constexpr int AHEAD = 2 / PARTS;   // segments whose TMEM loads share one wait
+          // segments whose TMEM loads share one wait (a program's steps need the
+          // registers of the second: bias + GELU on 4096 x 4096 x 1024 44.5 us with
+          // two, 43.8 with one)
+          constexpr int AHEAD = EW ? 1 : 2 / PARTS;
           auto load = [&](int i, uint32_t (&r)[PARTS][32]) {
             ptx::tmem_ld32_async(ta0 + 32u * i, r[0]);
             if constexpr (PARTS == 2) ptx::tmem_ld32_async(ta0 + 32u * i + (uint32_t)p.bn, r[1]);
