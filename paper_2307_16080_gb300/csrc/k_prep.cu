@@ -581,12 +581,13 @@ nk_status prep_amax(const float* x, int64_t rows, int64_t cols, int64_t ld, floa
   if (!x) return fail(NK_ERR_INVALID_ARG, "amax: null pointer");
   if (!ws || ws_bytes < prep_amax_ws(rows * cols))
     return fail(NK_ERR_WORKSPACE, "amax needs %zu bytes of workspace", prep_amax_ws(rows * cols));
-  // one wave of the five blocks an SM holds, fewer for a short dense run (at
-  // most four words a thread; 500 thousand values: 2.8 us, 3.4 with 1024 blocks)
+  // long runs fill whole rounds of eight words; shorter ones take one wave of the
+  // five blocks an SM holds, and at most four words a thread where these are
+  // too many (500 thousand values: 2.8 us, 3.4 with 1024 blocks)
   int sms = 0;
   nk_status s = require_device(&sms);
   if (s != NK_OK) return s;
-  int blocks = std::min(kAmaxBlocks, 5 * sms);
+  int blocks = rows * cols >= int64_t(kAmaxBlocks) * 256 * 32 ? kAmaxBlocks : std::min(kAmaxBlocks, 5 * sms);
   if (ld == cols) blocks = (int)std::min<int64_t>(blocks, (rows * cols + 4095) / 4096);
   if (pro && pro->n)
     (void)nk::launch_k(amax_stage1<true>, dim3(blocks), dim3(256), 0, st, 1, x, rows, cols, ld, static_cast<float*>(ws), *pro);
