@@ -181,10 +181,12 @@ static __device__ __forceinline__ float ew_step(int op, float x, float a, float 
 // program is present, and the plain paths carry no extra code.
 static __device__ __noinline__ float ew_run(const EwProg& e, float x, int64_t off) {
   for (int i = 0; i < e.n; ++i) {
-    const int op = e.op[i];
-    if (op == NK_EW_MUL) x = __fmul_rn(x, e.t[i][off]);
-    else if (op == NK_EW_ADD) x = __fadd_rn(x, e.t[i][off]);
-    else x = ew_step(op, x, e.a[i], e.b[i]);
+    const float a = e.a[i], b = e.b[i];
+    switch (e.op[i]) {
+      case NK_EW_MUL: x = __fmul_rn(x, e.t[i][off]); break;
+      case NK_EW_ADD: x = __fadd_rn(x, e.t[i][off]); break;
+      default: x = ew_step(e.op[i], x, a, b);
+    }
   }
   return x;
 }
